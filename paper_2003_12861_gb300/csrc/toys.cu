@@ -565,25 +565,90 @@ __global__ void __launch_bounds__(32 * kGenWarps, 7) events_kernel(
   }
 }
 
-// Per-set 64-bin histogram, one block per set.
-__global__ void hist64_kernel(const __grid_constant__ Columns cols, int col, const int64_t* __restrict__ offsets,
-                              double lo, double scale, float* __restrict__ out) {
-  __shared__ int bins[64];
-  const int s = blockIdx.x;
-  if (threadIdx.x < 64) bins[threadIdx.x] = 0;
+// Per-set 64-bin histogram: bin = floor((x - lo) scale) in FP64, clamped to
+// [0, 63].  Bound by the FP64 unit when taken literally (a conversion, a
+// subtraction, a product and a floor per event, 64 cycles each), so the bin is
+// taken in float where the float coordinate is further than `reach` (in bins)
+// from the next bin edge, which is its largest distance from the FP64 one for
+// an x in [lo - span, hi + span]; other x, NaN and infinities among them, take
+// the FP64 expression (1024 sets, 2.4e7 events: 305 -> 72 us).  `split` blocks share a set's events; with several,
+// they add their counts to the integers that the caller's output holds in the
+// meantime (hist64_norm_kernel turns them into fractions).
+constexpr int kHistThreads = 256, kHistCopies = 16;
+// Out of line: inlined, the compiler would compute the FP64 bin of every
+// event and select.
+__device__ __noinline__ int hist_bin_fp64(double x, double lo, double scale) {
+  return (int)floor(__dmul_rn(__dsub_rn(x, lo), scale));
+}
+__device__ __forceinline__ int hist_bin(double x, float xf, double lo, double scale, float lof, float scalef,
+                                        float reach) {
+  const float t = __fmul_rn(__fsub_rn(xf, lof), scalef);
+  const float b = floorf(t), f = __fsub_rn(t, b);
+  int bin;
+  if (f > reach && f < 1.0f - reach && t > -64.0f && t < 128.0f) bin = (int)b;
+  else bin = hist_bin_fp64(x, lo, scale);
+  return min(63, max(0, bin));
+}
+// The float nearest below |x| (from the bits: the FP64-to-float conversion
+// runs on the FP64 unit); zero for what is below the float range, infinite above.
+__device__ __forceinline__ float hist_float(double x) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int ex = (int)((h >> 20) & 0x7ffu) - 896;
+  const uint32_t mag = ex <= 0 ? 0u : ex >= 255 ? 0x7f800000u : ((uint32_t)ex << 23) | ((h & 0xfffffu) << 3) | (l >> 29);
+  return __uint_as_float((h & 0x80000000u) | mag);
+}
+template <bool kF32>
+__global__ void __launch_bounds__(kHistThreads) hist64_kernel(const void* __restrict__ colp,
+                                                              const int64_t* __restrict__ offsets, double lo,
+                                                              double scale, float lof, float scalef, float reach,
+                                                              int split, float* __restrict__ out) {
+  // 16 copies of the 64 counters, a lane's copy interleaved over the banks:
+  // a peaked column puts many of a warp's events into one bin
+  __shared__ int bins[64 * kHistCopies];
+  const int s = blockIdx.x / split, part = blockIdx.x % split, tid = threadIdx.x;
+  for (int i = tid; i < 64 * kHistCopies; i += kHistThreads) bins[i] = 0;
   __syncthreads();
-  const int64_t b0 = offsets[s], b1 = offsets[s + 1];
-  for (int64_t e = b0 + threadIdx.x; e < b1; e += blockDim.x) {
-    const double xv = cols.is_f32[col] ? (double)((const float*)cols.ptr[col])[e] : ((const double*)cols.ptr[col])[e];
-    int b = (int)floor(__dmul_rn(__dsub_rn(xv, lo), scale));
-    b = min(63, max(0, b));
-    atomicAdd(&bins[b], 1);
+  const int64_t b0 = offsets[s], b1 = offsets[s + 1], n = b1 - b0;
+  const int64_t e1 = b0 + n * (part + 1) / split;
+  int* mine = bins + tid % kHistCopies;
+  int64_t e = b0 + n * part / split + tid;
+  constexpr int kU = 8;  // loads in flight per thread
+  for (; e + (kU - 1) * kHistThreads < e1; e += kU * kHistThreads) {
+    if constexpr (kF32) {  // (an FP32 column widens only where FP64 decides)
+      float x[kU];
+#pragma unroll
+      for (int i = 0; i < kU; ++i) x[i] = __ldg((const float*)colp + e + i * kHistThreads);
+#pragma unroll
+      for (int i = 0; i < kU; ++i)
+        atomicAdd(mine + kHistCopies * hist_bin((double)x[i], x[i], lo, scale, lof, scalef, reach), 1);
+    } else {
+      double x[kU];
+#pragma unroll
+      for (int i = 0; i < kU; ++i) x[i] = __ldg((const double*)colp + e + i * kHistThreads);
+#pragma unroll
+      for (int i = 0; i < kU; ++i)
+        atomicAdd(mine + kHistCopies * hist_bin(x[i], hist_float(x[i]), lo, scale, lof, scalef, reach), 1);
+    }
+  }
+  for (; e < e1; e += kHistThreads) {
+    const double x = kF32 ? (double)__ldg((const float*)colp + e) : __ldg((const double*)colp + e);
+    const float xf = kF32 ? __ldg((const float*)colp + e) : hist_float(x);
+    atomicAdd(mine + kHistCopies * hist_bin(x, xf, lo, scale, lof, scalef, reach), 1);
   }
   __syncthreads();
-  if (threadIdx.x < 64) {
-    const int64_t n = b1 - b0;
-    out[(size_t)s * 64 + threadIdx.x] = n > 0 ? (float)((double)bins[threadIdx.x] / (double)n) : 0.0f;
+  if (tid < 64) {
+    int c = 0;
+    for (int i = 0; i < kHistCopies; ++i) c += bins[tid * kHistCopies + (i + tid) % kHistCopies];
+    float* o = out + (size_t)s * 64 + tid;
+    if (split == 1) *o = n > 0 ? (float)((double)c / (double)n) : 0.0f;
+    else if (c) atomicAdd(reinterpret_cast<int*>(o), c);
   }
+}
+__global__ void hist64_norm_kernel(const int64_t* __restrict__ offsets, int n_sets, float* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)n_sets * 64) return;
+  const int64_t n = offsets[i / 64 + 1] - offsets[i / 64];
+  out[i] = n > 0 ? (float)((double)__float_as_int(out[i]) / (double)n) : 0.0f;
 }
 
 // Appends the float filter's terms of the factor at node `root`, from term
@@ -804,15 +869,33 @@ rf_status rf_hist64(const rf_model* m, const rf_data* d, int32_t col, float* d_o
     set_error("rf_hist64: bad argument");
     return RF_E_INVALID;
   }
-  Columns c{};
-  for (int i = 0; i < d->n_obs; ++i) {
-    c.ptr[i] = d->cols[i];
-    c.is_f32[i] = d->dtype[i] == RF_F32;
+  const cudaStream_t st = (cudaStream_t)stream;
+  const double lo = m->m.obs_lo[col], hi = m->m.obs_hi[col], scale = 64.0 / (hi - lo);
+  // x, lo and scale as floats, the difference and the product: at most 2^-23
+  // of |x| + |lo|, in bins, and 2^-22 of the coordinate (below 128); four times
+  // that (beyond 0.5, every event takes the FP64 expression).
+  const double far = std::max(std::fabs(lo), std::fabs(hi)) + (hi - lo);
+  const float reach = (float)std::min(1.0, 4.0 * (2.0 * far * scale * 0x1p-23 + 128.0 * 0x1p-22));
+  // Blocks per set: 8 resident blocks an SM fill the GPU; a block takes at
+  // least 16384 events (64 a thread), below which a second one gains nothing.
+  const int64_t per_set = (d->n_events + d->n_sets - 1) / d->n_sets;
+  const int64_t most = std::max<int64_t>(1, 8 * (int64_t)sm_count() / d->n_sets);
+  const int split = (int)std::max<int64_t>(1, std::min(most, per_set / 16384));
+  const int64_t* off = (const int64_t*)d->offsets_dev.p;
+  if (split > 1 &&
+      !cuda_ok(cudaMemsetAsync(d_out, 0, sizeof(float) * 64 * (size_t)d->n_sets, st), "rf_hist64 reset"))
+    return RF_E_CUDA;
+  note_launches(1, st);
+  if (d->dtype[col] == RF_F32)
+    hist64_kernel<true><<<d->n_sets * split, kHistThreads, 0, st>>>(d->cols[col], off, lo, scale, (float)lo,
+                                                                   (float)scale, reach, split, d_out);
+  else
+    hist64_kernel<false><<<d->n_sets * split, kHistThreads, 0, st>>>(d->cols[col], off, lo, scale, (float)lo,
+                                                                    (float)scale, reach, split, d_out);
+  if (split > 1) {
+    note_launches(1, st);
+    hist64_norm_kernel<<<(d->n_sets * 64 + 255) / 256, 256, 0, st>>>(off, d->n_sets, d_out);
   }
-  const double lo = m->m.obs_lo[col], hi = m->m.obs_hi[col];
-  note_launches(1, (cudaStream_t)stream);
-  hist64_kernel<<<d->n_sets, 256, 0, (cudaStream_t)stream>>>(c, col, (const int64_t*)d->offsets_dev.p, lo,
-                                                            64.0 / (hi - lo), d_out);
   return cuda_ok(cudaGetLastError(), "rf_hist64 launch") ? RF_OK : RF_E_CUDA;
 }
 
