@@ -14,9 +14,16 @@
 // parameter k: a normfactor or normsys on sample s contributes dlog(factor)
 // / dtheta_k sum_i w nu_s[i], a histosys F_s sum_i w (a_i + b_i g').
 //
-// One block per dataset (persistent over datasets), every sum in a fixed
-// order (each thread's bins / samples / modifiers in index order, a fixed
-// tree across threads), so results do not depend on the launch.  The two
+// (One block per dataset, each reading every coefficient for itself and waiting
+// for it, took 490 us for one dataset of the 28-channel model and 1500 us for
+// 1024; this takes 76 and 856 us: the float-float loops 0.29 ms each, at about
+// 60 % of the FP32 pipe's rate, the bins' FP64 division and logarithm 0.13 ms.)
+// A pass is five chained kernels over (dataset, work) grids -- parameters and
+// sample factors, entry rates, bins, weighted sums, gradient and NLL -- so one
+// dataset fills as many SMs as its work can, and many datasets share every
+// coefficient load (four datasets a thread).  Every sum has a fixed order
+// (samples, bins and modifiers in index order, fixed trees), so results do not
+// depend on the launch or on the other datasets.  The two
 // loops that carry nearly all the multiply-adds -- the entries' histosys
 // sums and the histosys modifiers' weighted coefficient sums -- and the
 // samples' weighted sums run in float-float on the FP32 pipe (ff.cuh: FP64
@@ -40,14 +47,24 @@ namespace {
 constexpr int kBinnedThreads = 256;
 constexpr int kMaxBinnedBins = 8192, kMaxBinnedSamples = 2048;
 
-// Dynamic shared memory of the kernels (8-byte slots): theta, F and Ssum per
-// sample, W per bin (a float pair), one partial sum per thread, g and g' per
-// parameter, then theta, g and F as float pairs.
+// The largest model: this many bytes have to fit a block's shared memory (the
+// expected-counts kernel's theta, g, g' and F fit in them too).
 size_t binned_smem(int n_params, int n_samples, int n_bins) {
   return sizeof(double) * (5 * (size_t)n_params + 3 * (size_t)n_samples + (size_t)n_bins + kBinnedThreads);
 }
 
 enum ModKind : int32_t { MOD_NORMFACTOR = 0, MOD_NORMSYS = 1, MOD_HISTOSYS = 2 };
+
+// A factor modifier of a sample and a modifier of a parameter (normsys: a, b of
+// log eta = a alpha + b g(alpha)).
+struct FactorRec {
+  int32_t param, kind;
+  double a, b;
+};
+struct GradRec {
+  int32_t kind, sample, hs, pad;
+  double a, b;
+};
 
 struct BinnedDev {
   int32_t n_bins, n_samples, n_params, n_mods, n_entries, n_hs;
@@ -56,27 +73,17 @@ struct BinnedDev {
   const int32_t* eofs;        // per sample: its first (sample, bin) entry; entries run sample by sample
   const int32_t* esample;     // per entry: its sample
   const double* nominal;      // per entry
-  const int32_t* smod_start;  // per sample: its normfactor / normsys modifiers (CSR, modifier order)
-  const int32_t* smod;
+  const int32_t* smod_start;  // per sample: its normfactor / normsys modifiers (CSR, modifier order; `factor`)
   const int32_t* shs_start;   // per sample: its histosys modifiers (CSR, modifier order), as indices
   const int32_t* shs;         //   into the histosys arrays below
-  const int32_t* kind;        // per modifier
-  const int32_t* param;
-  const int32_t* msample;
-  const int32_t* mhs;         // per modifier: its histosys index, or -1
-  const double* ns_a;         // normsys: a, b of log eta = a alpha + b g(alpha)
-  const double* ns_b;
-  const int32_t* hs_param;    // per histosys: parameter, sample
-  const int32_t* hs_sample;
+  const int32_t* hs_param;    // per histosys: its parameter
   const int64_t* hs_ofs;      // per histosys: a_i then b_i, nb each, in `coef`
   const double* coef;
   // The same coefficients transposed per sample for the weighted sums:
   // sample s's histosys j (its j-th in shs order) at local bin i sits at
-  // tbase[s] + i * (histosys of s) + j, in coef_a and coef_b.
+  // tbase[s] + i * (histosys of s) + j, in coef_af and coef_bf.
   const int64_t* tbase;
   const int32_t* g_sample;    // per position in shs: its sample
-  const double* coef_a;
-  const double* coef_b;
   // The nominal rates and the histosys coefficients again as float pairs
   // (same indexing), for the float-float loops.
   const float2* nominal_f;
@@ -87,39 +94,58 @@ struct BinnedDev {
   const float2* coef_bf;
   const int32_t* bin_start;   // per bin: its entries (CSR, sample order)
   const int32_t* bin_entry;
-  const int32_t* pmod_start;  // per parameter: its modifiers (CSR, modifier order)
-  const int32_t* pmod;
+  const int32_t* pmod_start;  // per parameter: its modifiers (CSR, modifier order; `grad`)
   const int32_t* constrained;
+  // The modifiers as records in the order they are summed.
+  const FactorRec* factor;
+  const GradRec* grad;
 };
 
-// theta, g(theta) and g'(theta) into smem (once per parameter and dataset:
+// The intermediate results of a pass for up to `cap` datasets, dataset-major.
+struct BinnedScratch {
+  float4* pt;      // per parameter: theta and g as float pairs
+  double* dgk;     // g'
+  double* F;       // per sample: its factor, the same as a pair, sum_i w nu_s[i]
+  float2* Ff;
+  double* Ssum;
+  float2* nu_e;    // per entry
+  float2* W;       // per bin: weight, Poisson term
+  double* term;
+  double* T;       // per histosys: sum_i w (a_i + b_i g')
+};
+
+__device__ __forceinline__ ff ld_pair(const float2* p) {
+  const float2 v = __ldg(p);
+  return {v.x, v.y};
+}
+__device__ __forceinline__ ff as_ff(double v) { return ff_from_double(v); }
+
+// theta and g(theta) into smem (once per parameter and dataset:
 // an FP64 comparison per term would occupy the FP64 unit as long as the
 // multiply-add itself), then the sample factors F: the normfactors times
 // one exponential of the normsys exponents' sum.
 __device__ __forceinline__ void sample_factors(const BinnedDev& m, const double* th_g, double* th, double* gk,
-                                               double* dgk, double* F) {
+                                               double* F) {
   for (int k = threadIdx.x; k < m.n_params; k += kBinnedThreads) {
     const double a = th_g[k];
     th[k] = a;
     const bool in = fabs(a) <= 1.0;
     gk[k] = in ? a * a : 2.0 * fabs(a) - 1.0;
-    dgk[k] = in ? 2.0 * a : (a > 0.0 ? 2.0 : -2.0);
   }
   __syncthreads();
   for (int s = threadIdx.x; s < m.n_samples; s += kBinnedThreads) {
     double f = 1.0, le = 0.0;
     for (int j = m.smod_start[s]; j < m.smod_start[s + 1]; ++j) {
-      const int md = m.smod[j], k = m.param[md];
-      if (m.kind[md] == MOD_NORMFACTOR) f *= th[k];
-      else le = fma(m.ns_b[md], gk[k], fma(m.ns_a[md], th[k], le));
+      const FactorRec r = m.factor[j];
+      if (r.kind == MOD_NORMFACTOR) f *= th[r.param];
+      else le = fma(r.b, gk[r.param], fma(r.a, th[r.param], le));
     }
     F[s] = le != 0.0 ? f * exp(le) : f;
   }
   __syncthreads();
 }
 
-// nu of every (sample, bin) entry: consecutive threads take consecutive
-// bins of a sample, so its histosys coefficients are read coalesced.
+// nu of every (sample, bin) entry in FP64 (for the expected counts).
 __device__ __forceinline__ void entry_rates(const BinnedDev& m, const double* th, const double* gk, const double* F,
                                             double* nu_e) {
   for (int e = threadIdx.x; e < m.n_entries; e += kBinnedThreads) {
@@ -134,136 +160,250 @@ __device__ __forceinline__ void entry_rates(const BinnedDev& m, const double* th
   }
 }
 
-__device__ __forceinline__ ff ld_pair(const float2* p) {
-  const float2 v = __ldg(p);
-  return {v.x, v.y};
-}
-__device__ __forceinline__ ff as_ff(double v) { return ff_from_double(v); }
-
-// The same rates in float-float from the pairs' copies of the constants:
-// thf, gkf, Ff = theta, g, F as pairs.
-__device__ __forceinline__ void entry_rates_ff(const BinnedDev& m, const ff* thf, const ff* gkf, const ff* Ff,
-                                               ff* nu_e) {
-  for (int e = threadIdx.x; e < m.n_entries; e += kBinnedThreads) {
-    const int s = m.esample[e], i = e - m.eofs[s], n = m.nb[s];
-    ff shape = ld_pair(m.nominal_f + e);
-    const int j1 = m.shs_start[s + 1];
-#pragma unroll 4
-    for (int j = m.shs_start[s]; j < j1; ++j) {
-      const int k = __ldg(m.shs_k + j);
-      const float2* c = m.coef_f + __ldg(m.shs_ofs + j) + i;
-      shape = ff_fma(ld_pair(c + n), gkf[k], ff_fma(ld_pair(c), thf[k], shape));
-    }
-    nu_e[e] = ff_mul(Ff[s], shape);
-  }
+// Each kernel of a pass is a programmatic dependent of the one before: it is
+// scheduled while that runs and waits here for its results (which it then
+// reads with plain loads: the read-only path may not see them).
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// out[set]: NLL then gradient (1 + n_params); flags[set]: 1 if some bin has
-// nu <= 0 (NLL +inf).  scratch: per block n_entries (entry rates) +
-// n_hs (histosys sums) doubles.
-// sets: null, or the dataset (row of counts) of each of the n_sets points.
-__global__ void __launch_bounds__(kBinnedThreads) binned_kernel(const BinnedDev m, int n_sets, const int32_t* sets,
-                                                                 const double* counts, const double* theta,
-                                                                 double* out, int32_t* flags, double* scratch) {
+// Step 1: block (set, chunk of samples).  theta, g, g' of the set (all blocks
+// need them, chunk 0 stores them), then the chunk's sample factors: the
+// normfactors times one exponential of the normsys exponents' sum.
+constexpr int kPrepThreads = 128;
+__global__ void __launch_bounds__(kPrepThreads) binned_prep_kernel(const BinnedDev m, const BinnedScratch w,
+                                                                   const double* theta, int per_block,
+                                                                   int32_t* flags) {
   extern __shared__ double smem[];
   double* th = smem;
-  double* F = th + m.n_params;
-  double* Ssum = F + m.n_samples;
-  ff* W = reinterpret_cast<ff*>(Ssum + m.n_samples);
-  double* part = reinterpret_cast<double*>(W + m.n_bins);
-  double* gk = part + kBinnedThreads;
-  double* dgk = gk + m.n_params;
-  ff* thf = reinterpret_cast<ff*>(dgk + m.n_params);
-  ff* gkf = thf + m.n_params;
-  ff* Ff = gkf + m.n_params;
-  __shared__ int bad;
-  const int tid = threadIdx.x;
-  ff* nu_e = reinterpret_cast<ff*>(scratch + (size_t)blockIdx.x * (m.n_entries + m.n_hs));
-  double* T = reinterpret_cast<double*>(nu_e + m.n_entries);
-  for (int set = blockIdx.x; set < n_sets; set += gridDim.x) {
-    const double* n = counts + (size_t)(sets ? sets[set] : set) * m.n_bins;
-    if (tid == 0) bad = 0;
-    sample_factors(m, theta + (size_t)set * m.n_params, th, gk, dgk, F);
-    for (int k = tid; k < m.n_params; k += kBinnedThreads) {
-      thf[k] = as_ff(th[k]);
-      gkf[k] = as_ff(gk[k]);
+  double* gk = th + m.n_params;
+  chain_wait();
+  const int set = blockIdx.y;
+  const double* th_g = theta + (size_t)set * m.n_params;
+  for (int k = threadIdx.x; k < m.n_params; k += kPrepThreads) {
+    const double a = th_g[k];
+    const bool in = fabs(a) <= 1.0;
+    const double g = in ? a * a : 2.0 * fabs(a) - 1.0;
+    th[k] = a;
+    gk[k] = g;
+    if (blockIdx.x == 0) {
+      const ff t = as_ff(a), u = as_ff(g);
+      w.pt[(size_t)set * m.n_params + k] = make_float4(t.hi, t.lo, u.hi, u.lo);
+      w.dgk[(size_t)set * m.n_params + k] = in ? 2.0 * a : (a > 0.0 ? 2.0 : -2.0);
     }
-    for (int s = tid; s < m.n_samples; s += kBinnedThreads) Ff[s] = as_ff(F[s]);
-    __syncthreads();
-    entry_rates_ff(m, thf, gkf, Ff, nu_e);
-    __syncthreads();
-    // bins: expected count, weight 1 - n/nu, the Poisson term
-    double acc = 0.0;
-    for (int b = tid; b < m.n_bins; b += kBinnedThreads) {
-      ff nf = {0.0f, 0.0f};
-      const int j1 = m.bin_start[b + 1];
-#pragma unroll 4
-      for (int j = m.bin_start[b]; j < j1; ++j) nf = ff_add(nf, nu_e[__ldg(m.bin_entry + j)]);
-      const double nu = ff_to_double(nf);
-      if (!(nu > 0.0) || !isfinite(nu)) {
-        bad = 1;
-        W[b] = {0.0f, 0.0f};
-        continue;
-      }
-      W[b] = as_ff(1.0 - n[b] / nu);
-      acc += nu - (n[b] != 0.0 ? n[b] * log(nu) : 0.0);
-    }
-    part[tid] = acc;
-    __syncthreads();
-    // per sample sum_i w nu_s[i]; per histosys sum_i w (a_i + b_i g')
-    for (int s = tid; s < m.n_samples; s += kBinnedThreads) {
-      ff a = {0.0f, 0.0f};
-      const int nbs = m.nb[s], b0 = m.bin0[s], e0 = m.eofs[s];
-#pragma unroll 4
-      for (int i = 0; i < nbs; ++i) ff_acc_mul(a, W[b0 + i], nu_e[e0 + i]);
-      Ssum[s] = ff_to_double(a);
-    }
-    // (a thread each, bins in order; consecutive threads read consecutive
-    // coefficients of the transposed layout)
-    for (int g = tid; g < m.n_hs; g += kBinnedThreads) {
-      const int s = m.g_sample[g], h = m.shs[g];
-      const int nh = m.shs_start[s + 1] - m.shs_start[s], j = g - m.shs_start[s];
-      const float2* ca = m.coef_af + m.tbase[s] + j;
-      const float2* cb = m.coef_bf + m.tbase[s] + j;
-      const ff* w = W + m.bin0[s];
-      ff ta = {0.0f, 0.0f}, tb = {0.0f, 0.0f};
-      const int nbs = m.nb[s];
-#pragma unroll 4
-      for (int i = 0; i < nbs; ++i) {
-        ff_acc_mul(ta, w[i], ld_pair(ca + (size_t)i * nh));
-        ff_acc_mul(tb, w[i], ld_pair(cb + (size_t)i * nh));
-      }
-      T[h] = fma(dgk[m.hs_param[h]], ff_to_double(tb), ff_to_double(ta));
-    }
-    // NLL: the threads' partial sums by a fixed tree
-    for (int o = kBinnedThreads / 2; o > 0; o >>= 1) {
-      __syncthreads();
-      if (tid < o) part[tid] += part[tid + o];
-    }
-    __syncthreads();
-    double* o = out + (size_t)set * (1 + m.n_params);
-    // gradient: each parameter's modifiers in order, then its constraint
-    for (int k = tid; k < m.n_params; k += kBinnedThreads) {
-      double g = 0.0;
-      const double a = th[k];
-      for (int j = m.pmod_start[k]; j < m.pmod_start[k + 1]; ++j) {
-        const int md = m.pmod[j], s = m.msample[md];
-        if (m.kind[md] == MOD_NORMFACTOR) g += Ssum[s] / a;
-        else if (m.kind[md] == MOD_NORMSYS) g += Ssum[s] * fma(m.ns_b[md], dgk[k], m.ns_a[md]);
-        else g += F[s] * T[m.mhs[md]];
-      }
-      if (m.constrained[k]) g += a;
-      o[1 + k] = g;
-    }
-    if (tid == 0) {
-      double c = 0.0;
-      for (int k = 0; k < m.n_params; ++k)
-        if (m.constrained[k]) c += 0.5 * th[k] * th[k];
-      o[0] = bad ? INFINITY : part[0] + c;
-      flags[set] = bad;
-    }
-    __syncthreads();
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) flags[set] = 0;
+  __syncthreads();
+  const int s1 = min(m.n_samples, (int)(blockIdx.x + 1) * per_block);
+  for (int s = blockIdx.x * per_block + threadIdx.x; s < s1; s += kPrepThreads) {
+    double f = 1.0, le = 0.0;
+    const int j1 = m.smod_start[s + 1];
+#pragma unroll 4
+    for (int j = m.smod_start[s]; j < j1; ++j) {
+      const FactorRec r = m.factor[j];
+      if (r.kind == MOD_NORMFACTOR) f *= th[r.param];
+      else le = fma(r.b, gk[r.param], fma(r.a, th[r.param], le));
+    }
+    const double F = le != 0.0 ? f * exp(le) : f;
+    w.F[(size_t)set * m.n_samples + s] = F;
+    const ff p = as_ff(F);
+    w.Ff[(size_t)set * m.n_samples + s] = make_float2(p.hi, p.lo);
+  }
+}
+
+// Step 2: nu of every (sample, bin) entry, a thread per entry for kSets
+// datasets: consecutive threads take consecutive bins of a sample, so its
+// histosys coefficients are read coalesced, once for the kSets datasets.
+constexpr int kBinnedThreads2 = 128;
+template <int kSets>
+__global__ void __launch_bounds__(kBinnedThreads2) binned_rates_kernel(const BinnedDev m, const BinnedScratch w,
+                                                                       int n_sets) {
+  chain_wait();
+  const int e = blockIdx.x * kBinnedThreads2 + threadIdx.x;
+  if (e >= m.n_entries) return;
+  const int set0 = blockIdx.y * kSets;
+  const float4* pt[kSets];
+#pragma unroll
+  for (int t = 0; t < kSets; ++t) pt[t] = w.pt + (size_t)min(set0 + t, n_sets - 1) * m.n_params;
+  const int s = m.esample[e], i = e - m.eofs[s], n = m.nb[s], j1 = m.shs_start[s + 1];
+  ff shape[kSets];
+  const ff nom = ld_pair(m.nominal_f + e);
+#pragma unroll
+  for (int t = 0; t < kSets; ++t) shape[t] = nom;
+#pragma unroll 4
+  for (int j = m.shs_start[s]; j < j1; ++j) {
+    const int k = __ldg(m.shs_k + j);
+    const float2* c = m.coef_f + __ldg(m.shs_ofs + j) + i;
+    const ff c0 = ld_pair(c), c1 = ld_pair(c + n);
+#pragma unroll
+    for (int t = 0; t < kSets; ++t) {
+      const float4 q = pt[t][k];
+      shape[t] = ff_fma(c1, ff{q.z, q.w}, ff_fma(c0, ff{q.x, q.y}, shape[t]));
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < kSets; ++t)
+    if (set0 + t < n_sets) {
+      const float2 f = w.Ff[(size_t)(set0 + t) * m.n_samples + s];
+      const ff v = ff_mul(ff{f.x, f.y}, shape[t]);
+      w.nu_e[(size_t)(set0 + t) * m.n_entries + e] = make_float2(v.hi, v.lo);
+    }
+}
+
+// Step 3: per bin the expected count (samples in order), the weight 1 - n/nu
+// and the Poisson term.  sets: null, or the row of counts of each dataset.
+__global__ void __launch_bounds__(kBinnedThreads2) binned_bins_kernel(const BinnedDev m, const BinnedScratch w,
+                                                                      const int32_t* sets, const double* counts,
+                                                                      int32_t* flags) {
+  chain_wait();
+  const int b = blockIdx.x * kBinnedThreads2 + threadIdx.x, set = blockIdx.y;
+  if (b >= m.n_bins) return;
+  const double n = counts[(size_t)(sets ? sets[set] : set) * m.n_bins + b];
+  const float2* nu_e = w.nu_e + (size_t)set * m.n_entries;
+  ff nf = {0.0f, 0.0f};
+  const int j1 = m.bin_start[b + 1];
+#pragma unroll 4
+  for (int j = m.bin_start[b]; j < j1; ++j) {
+    const float2 v = nu_e[__ldg(m.bin_entry + j)];
+    nf = ff_add(nf, ff{v.x, v.y});
+  }
+  const double nu = ff_to_double(nf);
+  float2 wt = make_float2(0.0f, 0.0f);
+  double term = 0.0;
+  if (!(nu > 0.0) || !isfinite(nu)) {
+    flags[set] = 1;
+  } else {
+    const ff p = as_ff(1.0 - n / nu);
+    wt = make_float2(p.hi, p.lo);
+    term = nu - (n != 0.0 ? n * log(nu) : 0.0);
+  }
+  w.W[(size_t)set * m.n_bins + b] = wt;
+  w.term[(size_t)set * m.n_bins + b] = term;
+}
+
+// Step 4: per histosys sum_i w (a_i + b_i g') and per sample sum_i w nu_s[i],
+// for kSets datasets.  A block takes 32 of them (threads along them, so
+// consecutive threads read consecutive coefficients of the transposed layout)
+// times four quarters of the sample's bins (one chain of dependent
+// multiply-adds a quarter as long), added in order at the end; a warp's
+// weights are those of one or two samples.
+constexpr int kQuarters = kBinnedThreads2 / 32;
+template <int kSets>
+__global__ void __launch_bounds__(kBinnedThreads2) binned_sums_kernel(const BinnedDev m, const BinnedScratch w,
+                                                                      int n_sets) {
+  __shared__ float4 part[kQuarters - 1][kSets][32];
+  chain_wait();
+  const int lane = threadIdx.x & 31, quarter = threadIdx.x >> 5, set0 = blockIdx.y * kSets;
+  const int id = blockIdx.x * 32 + lane, s = id < m.n_hs ? m.g_sample[id] : id - m.n_hs;
+  const bool hs = id < m.n_hs, any = s < m.n_samples;
+  ff ta[kSets], tb[kSets];
+#pragma unroll
+  for (int t = 0; t < kSets; ++t) ta[t] = tb[t] = {0.0f, 0.0f};
+  if (any) {
+    const int nbs = m.nb[s], i0 = nbs * quarter / kQuarters, i1 = nbs * (quarter + 1) / kQuarters;
+    const float2* W[kSets];
+#pragma unroll
+    for (int t = 0; t < kSets; ++t) W[t] = w.W + (size_t)min(set0 + t, n_sets - 1) * m.n_bins + m.bin0[s];
+    if (hs) {
+      const int j0 = m.shs_start[s], nh = m.shs_start[s + 1] - j0;
+      const float2* ca = m.coef_af + m.tbase[s] + (id - j0);
+      const float2* cb = m.coef_bf + m.tbase[s] + (id - j0);
+#pragma unroll 4
+      for (int i = i0; i < i1; ++i) {
+        const ff a = ld_pair(ca + (size_t)i * nh), b = ld_pair(cb + (size_t)i * nh);
+#pragma unroll
+        for (int t = 0; t < kSets; ++t) {
+          const float2 v = W[t][i];
+          ff_acc_mul(ta[t], ff{v.x, v.y}, a);
+          ff_acc_mul(tb[t], ff{v.x, v.y}, b);
+        }
+      }
+    } else {
+      const float2* nu[kSets];
+#pragma unroll
+      for (int t = 0; t < kSets; ++t) nu[t] = w.nu_e + (size_t)min(set0 + t, n_sets - 1) * m.n_entries + m.eofs[s];
+#pragma unroll 4
+      for (int i = i0; i < i1; ++i)
+#pragma unroll
+        for (int t = 0; t < kSets; ++t) {
+          const float2 v = W[t][i], e = nu[t][i];
+          ff_acc_mul(ta[t], ff{v.x, v.y}, ff{e.x, e.y});
+        }
+    }
+  }
+  if (quarter > 0)
+#pragma unroll
+    for (int t = 0; t < kSets; ++t) part[quarter - 1][t][lane] = make_float4(ta[t].hi, ta[t].lo, tb[t].hi, tb[t].lo);
+  __syncthreads();
+  if (quarter > 0 || !any) return;
+#pragma unroll
+  for (int t = 0; t < kSets; ++t) {
+    if (set0 + t >= n_sets) break;
+    for (int q = 0; q < kQuarters - 1; ++q) {
+      const float4 v = part[q][t][lane];
+      ta[t] = ff_add(ta[t], ff{v.x, v.y});
+      tb[t] = ff_add(tb[t], ff{v.z, v.w});
+    }
+    if (hs)
+      w.T[(size_t)(set0 + t) * m.n_hs + m.shs[id]] =
+          fma(w.dgk[(size_t)(set0 + t) * m.n_params + m.shs_k[id]], ff_to_double(tb[t]), ff_to_double(ta[t]));
+    else
+      w.Ssum[(size_t)(set0 + t) * m.n_samples + s] = ff_to_double(ta[t]);
+  }
+}
+
+// Step 5: out[set] = NLL, then gradient.  Block (0, set): the bins' terms and
+// the constraints summed, each by thread-strided sums and a fixed tree; the
+// others 16 parameters each, eight lanes a parameter: its modifiers lane by
+// lane, the lanes by butterfly, then its constraint.
+constexpr int kGradThreads = 128, kGradLanes = 8, kGradPer = kGradThreads / kGradLanes;
+__global__ void __launch_bounds__(kGradThreads) binned_grad_kernel(const BinnedDev m, const BinnedScratch w,
+                                                                   const double* theta, double* out,
+                                                                   const int32_t* flags) {
+  chain_wait();
+  const int set = blockIdx.y, tid = threadIdx.x;
+  const double* th = theta + (size_t)set * m.n_params;
+  double* o = out + (size_t)set * (1 + m.n_params);
+  if (blockIdx.x == 0) {
+    __shared__ double red[kGradThreads];
+    const double* term = w.term + (size_t)set * m.n_bins;
+    double t = 0.0, c = 0.0;
+#pragma unroll 4
+    for (int b = tid; b < m.n_bins; b += kGradThreads) t += term[b];
+    for (int k = tid; k < m.n_params; k += kGradThreads)
+      if (m.constrained[k]) c = fma(0.5 * th[k], th[k], c);
+    red[tid] = t + c;
+    for (int d = kGradThreads / 2; d > 0; d >>= 1) {
+      __syncthreads();
+      if (tid < d) red[tid] += red[tid + d];
+    }
+    if (tid == 0) o[0] = flags[set] ? INFINITY : red[0];
+    return;
+  }
+  const int k = (blockIdx.x - 1) * kGradPer + tid / kGradLanes, l = tid % kGradLanes;
+  double g = 0.0, a = 0.0;
+  if (k < m.n_params) {
+    const double* F = w.F + (size_t)set * m.n_samples;
+    const double* S = w.Ssum + (size_t)set * m.n_samples;
+    const double* T = w.T + (size_t)set * m.n_hs;
+    a = th[k];
+    const double dg = w.dgk[(size_t)set * m.n_params + k];
+    const int j1 = m.pmod_start[k + 1];
+#pragma unroll 4
+    for (int j = m.pmod_start[k] + l; j < j1; j += kGradLanes) {
+      const GradRec r = m.grad[j];
+      const double x = r.kind == MOD_HISTOSYS ? F[r.sample] : S[r.sample];
+      double y;
+      if (r.kind == MOD_HISTOSYS) y = T[r.hs];
+      else if (r.kind == MOD_NORMSYS) y = fma(r.b, dg, r.a);
+      else y = 1.0 / a;
+      g = fma(x, y, g);
+    }
+  }
+#pragma unroll
+  for (int d = kGradLanes / 2; d > 0; d >>= 1) g += __shfl_xor_sync(0xffffffffu, g, d);
+  if (k < m.n_params && l == 0) o[1 + k] = m.constrained[k] ? g + a : g;
 }
 
 // Expected counts nu_b per dataset (for generating toys).
@@ -274,10 +414,9 @@ __global__ void __launch_bounds__(kBinnedThreads) binned_expected_kernel(const B
   double* th = smem;
   double* F = th + m.n_params;
   double* gk = F + m.n_samples;
-  double* dgk = gk + m.n_params;
   double* nu_e = scratch + (size_t)blockIdx.x * (m.n_entries + m.n_hs);
   for (int set = blockIdx.x; set < n_sets; set += gridDim.x) {
-    sample_factors(m, theta + (size_t)set * m.n_params, th, gk, dgk, F);
+    sample_factors(m, theta + (size_t)set * m.n_params, th, gk, F);
     entry_rates(m, th, gk, F, nu_e);
     __syncthreads();
     for (int b = threadIdx.x; b < m.n_bins; b += kBinnedThreads) {
@@ -297,13 +436,14 @@ __global__ void __launch_bounds__(kBinnedThreads) binned_expected_kernel(const B
 
 struct rf_binned {
   int32_t n_bins = 0, n_samples = 0, n_params = 0, n_mods = 0, n_entries = 0, n_hs = 0;
-  rf::DevBuf bin0, nb, eofs, esample, nominal, smod_start, smod, shs_start, shs, kind, param, msample, mhs, ns_a,
-      ns_b, hs_param, hs_sample, hs_ofs, coef, tbase, g_sample, coef_a, coef_b, bin_start, bin_entry, pmod_start, pmod,
-      constrained, nominal_f, coef_f, coef_af, coef_bf, shs_k, shs_ofs;
-  rf::DevBuf scratch, counts, theta, out, flags, sets;
+  rf::DevBuf bin0, nb, eofs, esample, nominal, smod_start, shs_start, shs, hs_param, hs_ofs, coef, tbase, g_sample,
+      bin_start, bin_entry, pmod_start, constrained, nominal_f, coef_f, coef_af, coef_bf, shs_k, shs_ofs, factor, grad;
+  rf::DevBuf scratch, work, counts, theta, out, flags, sets;
   rf::HostBuf h_out, h_flags, h_theta, h_sets;
   rf::BinnedDev dev{};
-  int grid = 0;
+  rf::BinnedScratch ws{};
+  int grid = 0;  // blocks of the expected-counts kernel
+  int cap = 0;   // datasets a pass takes at once
   size_t smem = 0;
 };
 
@@ -317,13 +457,55 @@ bool upload(DevBuf& b, const std::vector<T>& v) {
   return v.empty() || cuda_ok(cudaMemcpy(b.p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice), "binned upload");
 }
 
+// Launches a kernel that begins with chain_wait(), as a programmatic dependent
+// of the stream's previous kernel.
+template <class... Params, class... Args>
+void launch_chained(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  note_launches(1, st);
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 rf_status launch_binned(rf_binned* m, int32_t n_sets, const double* d_counts, const double* d_theta, double* d_out,
                         int32_t* d_flags, cudaStream_t st, const int32_t* d_sets = nullptr) {
-  if (n_sets == 0) return RF_OK;
-  const int grid = std::min(n_sets, m->grid);
-  note_launches(1, st);
-  binned_kernel<<<grid, kBinnedThreads, m->smem, st>>>(m->dev, n_sets, d_sets, d_counts, d_theta, d_out, d_flags,
-                                                        (double*)m->scratch.p);
+  const BinnedDev& D = m->dev;
+  const int P = D.n_params;
+  for (int s0 = 0; s0 < n_sets; s0 += m->cap) {
+    const int n = std::min(n_sets - s0, m->cap);
+    const double* th = d_theta + (size_t)s0 * P;
+    const double* counts = d_sets ? d_counts : d_counts + (size_t)s0 * D.n_bins;
+    const int32_t* sets = d_sets ? d_sets + s0 : nullptr;
+    double* out = d_out + (size_t)s0 * (1 + P);
+    int32_t* flags = d_flags + s0;
+    // samples per block of step 1: 32 while that leaves SMs free (each block
+    // repeats the parameters' part), else a block per dataset
+    const int per_block = (int64_t)n * ((D.n_samples + 31) / 32) <= 2 * sm_count() ? 32 : D.n_samples;
+    auto blocks = [](int work, int threads) { return (unsigned)((work + threads - 1) / threads); };
+    launch_chained(binned_prep_kernel, dim3(blocks(D.n_samples, per_block), n), kPrepThreads,
+                   2 * sizeof(double) * (size_t)P, st, D, m->ws, th, per_block, flags);
+    // four datasets a thread (one load of a coefficient for the four) once the
+    // blocks still fill the GPU at that; one at a time else
+    const dim3 ge(blocks(D.n_entries, kBinnedThreads2)), gs(blocks(D.n_hs + D.n_samples, 32));
+    const bool four = (int64_t)ge.x * n >= 32 * (int64_t)sm_count();
+    const unsigned ny = four ? blocks(n, 4) : (unsigned)n;
+    launch_chained(four ? binned_rates_kernel<4> : binned_rates_kernel<1>, dim3(ge.x, ny), kBinnedThreads2, 0, st, D,
+                   m->ws, n);
+    launch_chained(binned_bins_kernel, dim3(blocks(D.n_bins, kBinnedThreads2), n), kBinnedThreads2, 0, st, D, m->ws,
+                   sets, counts, flags);
+    launch_chained(four ? binned_sums_kernel<4> : binned_sums_kernel<1>, dim3(gs.x, ny), kBinnedThreads2, 0, st, D,
+                   m->ws, n);
+    launch_chained(binned_grad_kernel, dim3(1 + blocks(P, kGradPer), n), kGradThreads, 0, st, D, m->ws, th, out,
+                   (const int32_t*)flags);
+  }
   return cuda_ok(cudaGetLastError(), "binned launch") ? RF_OK : RF_E_CUDA;
 }
 
@@ -358,7 +540,7 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   }
   std::vector<int32_t> kind(n_mods), param(n_mods), msample(n_mods), mhs(n_mods, -1);
   std::vector<double> ns_a(n_mods, 0.0), ns_b(n_mods, 0.0);
-  std::vector<int32_t> hs_param, hs_sample;
+  std::vector<int32_t> hs_param;
   std::vector<int64_t> hs_ofs;
   std::vector<double> coef;
   int64_t hd = 0;
@@ -390,7 +572,6 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
       const double *lo = hist_data + hd, *hi = hist_data + hd + n;
       mhs[j] = (int32_t)hs_param.size();
       hs_param.push_back(md.param);
-      hs_sample.push_back(md.sample);
       hs_ofs.push_back((int64_t)coef.size());
       for (int i = 0; i < n; ++i) coef.push_back(0.5 * (hi[i] - lo[i]));
       for (int i = 0; i < n; ++i) coef.push_back(0.5 * (hi[i] + lo[i]) - h[i]);
@@ -461,6 +642,13 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
     shs_ofs[j] = hs_ofs[shs[j]];
   }
   // float-pair copies: hi = the float nearest v, lo = the float nearest v - hi
+  std::vector<FactorRec> factor(smod.size());
+  for (size_t j = 0; j < smod.size(); ++j) factor[j] = FactorRec{param[smod[j]], kind[smod[j]], ns_a[smod[j]], ns_b[smod[j]]};
+  std::vector<GradRec> grad(pmod.size());
+  for (size_t j = 0; j < pmod.size(); ++j) {
+    const int md = pmod[j];
+    grad[j] = GradRec{kind[md], msample[md], mhs[md], 0, ns_a[md], ns_b[md]};
+  }
   auto pairs = [](const std::vector<double>& v) {
     std::vector<float2> f(v.size());
     for (size_t i = 0; i < v.size(); ++i) {
@@ -469,25 +657,21 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
     }
     return f;
   };
-  const bool ok = upload(m->shs_k, shs_k) && upload(m->shs_ofs, shs_ofs) &&
-                  upload(m->nominal_f, pairs(vnom)) && upload(m->coef_f, pairs(coef)) &&
+  const bool ok = upload(m->factor, factor) && upload(m->grad, grad) && upload(m->shs_k, shs_k) &&
+                  upload(m->shs_ofs, shs_ofs) && upload(m->nominal_f, pairs(vnom)) && upload(m->coef_f, pairs(coef)) &&
                   upload(m->coef_af, pairs(coef_a)) && upload(m->coef_bf, pairs(coef_b)) &&
                   upload(m->bin0, vb0) && upload(m->nb, vnb) && upload(m->eofs, eofs) && upload(m->esample, esample) &&
-                  upload(m->nominal, vnom) && upload(m->smod_start, smod_start) && upload(m->smod, smod) &&
-                  upload(m->shs_start, shs_start) && upload(m->shs, shs) && upload(m->kind, kind) &&
-                  upload(m->param, param) && upload(m->msample, msample) && upload(m->mhs, mhs) &&
-                  upload(m->ns_a, ns_a) && upload(m->ns_b, ns_b) && upload(m->hs_param, hs_param) &&
-                  upload(m->hs_sample, hs_sample) && upload(m->hs_ofs, hs_ofs) && upload(m->coef, coef) &&
-                  upload(m->tbase, tbase) && upload(m->g_sample, g_sample) && upload(m->coef_a, coef_a) &&
-                  upload(m->coef_b, coef_b) &&
+                  upload(m->nominal, vnom) && upload(m->smod_start, smod_start) && upload(m->shs_start, shs_start) &&
+                  upload(m->shs, shs) && upload(m->hs_param, hs_param) && upload(m->hs_ofs, hs_ofs) &&
+                  upload(m->coef, coef) && upload(m->tbase, tbase) && upload(m->g_sample, g_sample) &&
                   upload(m->bin_start, bin_start) && upload(m->bin_entry, bin_entry) &&
-                  upload(m->pmod_start, pmod_start) && upload(m->pmod, pmod) && upload(m->constrained, vcon);
+                  upload(m->pmod_start, pmod_start) && upload(m->constrained, vcon);
   m->smem = binned_smem(n_params, n_samples, n_bins);
   int dev_id = 0, max_optin = 0;
   cudaGetDevice(&dev_id);
   cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev_id);
   if (m->smem > (size_t)max_optin ||
-      !cuda_ok(cudaFuncSetAttribute(binned_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem),
+      !cuda_ok(cudaFuncSetAttribute(binned_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem),
                "binned smem") ||
       !cuda_ok(cudaFuncSetAttribute(binned_expected_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)m->smem),
@@ -497,11 +681,36 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
     return RF_E_INVALID;
   }
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, binned_kernel, kBinnedThreads, m->smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, binned_expected_kernel, kBinnedThreads, m->smem);
   m->grid = sm_count() * std::max(1, per_sm);
-  if (!ok || !m->scratch.ensure(sizeof(double) * (size_t)m->grid * (size_t)(m->n_entries + std::max(1, n_hs)))) {
+  // A pass's intermediate results: datasets in groups that need at most
+  // 256 MB (1024 at most, one at least).
+  const size_t P_ = (size_t)std::max(1, n_params), S_ = (size_t)n_samples, E_ = (size_t)total, B_ = (size_t)n_bins,
+               H_ = (size_t)std::max(1, n_hs);
+  const size_t per_set = 24 * P_ + 24 * S_ + 8 * E_ + 16 * B_ + 8 * H_;
+  m->cap = (int)std::max<size_t>(1, std::min<size_t>(1024, ((size_t)256 << 20) / per_set));
+  // (the expected counts' entry rates: per block n_entries + n_hs doubles)
+  if (!ok || !m->scratch.ensure(sizeof(double) * (size_t)m->grid * (E_ + H_)) ||
+      !m->work.ensure(per_set * (size_t)m->cap)) {
     delete m;
     return RF_E_OOM;
+  }
+  {
+    char* p = (char*)m->work.p;  // (16-byte items first)
+    auto take = [&](size_t bytes) {
+      char* q = p;
+      p += bytes * (size_t)m->cap;
+      return (void*)q;
+    };
+    m->ws.pt = (float4*)take(16 * P_);
+    m->ws.dgk = (double*)take(8 * P_);
+    m->ws.F = (double*)take(8 * S_);
+    m->ws.Ssum = (double*)take(8 * S_);
+    m->ws.Ff = (float2*)take(8 * S_);
+    m->ws.nu_e = (float2*)take(8 * E_);
+    m->ws.W = (float2*)take(8 * B_);
+    m->ws.term = (double*)take(8 * B_);
+    m->ws.T = (double*)take(8 * H_);
   }
   BinnedDev& D = m->dev;
   D.n_bins = n_bins;
@@ -516,23 +725,13 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   D.esample = (const int32_t*)m->esample.p;
   D.nominal = (const double*)m->nominal.p;
   D.smod_start = (const int32_t*)m->smod_start.p;
-  D.smod = (const int32_t*)m->smod.p;
   D.shs_start = (const int32_t*)m->shs_start.p;
   D.shs = (const int32_t*)m->shs.p;
-  D.kind = (const int32_t*)m->kind.p;
-  D.param = (const int32_t*)m->param.p;
-  D.msample = (const int32_t*)m->msample.p;
-  D.mhs = (const int32_t*)m->mhs.p;
-  D.ns_a = (const double*)m->ns_a.p;
-  D.ns_b = (const double*)m->ns_b.p;
   D.hs_param = (const int32_t*)m->hs_param.p;
-  D.hs_sample = (const int32_t*)m->hs_sample.p;
   D.hs_ofs = (const int64_t*)m->hs_ofs.p;
   D.coef = (const double*)m->coef.p;
   D.tbase = (const int64_t*)m->tbase.p;
   D.g_sample = (const int32_t*)m->g_sample.p;
-  D.coef_a = (const double*)m->coef_a.p;
-  D.coef_b = (const double*)m->coef_b.p;
   D.nominal_f = (const float2*)m->nominal_f.p;
   D.shs_k = (const int32_t*)m->shs_k.p;
   D.shs_ofs = (const int64_t*)m->shs_ofs.p;
@@ -542,8 +741,9 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   D.bin_start = (const int32_t*)m->bin_start.p;
   D.bin_entry = (const int32_t*)m->bin_entry.p;
   D.pmod_start = (const int32_t*)m->pmod_start.p;
-  D.pmod = (const int32_t*)m->pmod.p;
   D.constrained = (const int32_t*)m->constrained.p;
+  D.factor = (const FactorRec*)m->factor.p;
+  D.grad = (const GradRec*)m->grad.p;
   *out = m;
   return RF_OK;
 }
