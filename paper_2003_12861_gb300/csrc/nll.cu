@@ -759,13 +759,18 @@ __device__ __forceinline__ int warp_sum_int(int v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ Pair warp_merge(Pair p) {
+// Lane 0's butterfly sum (offsets 16, 8, 4, 2, 1) of two quantities whose
+// pairs are zero from lane m on: a merge with zeros changes nothing, so the
+// offsets >= m are left out; the two chains of FP64 additions overlap.
+__device__ __forceinline__ void warp_merge2(Pair& p, Pair& q, int m) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    Pair q{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.c, o)};
-    p = merge(p, q);
+    if (o >= m) continue;
+    const Pair a{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.c, o)};
+    const Pair b{__shfl_xor_sync(0xffffffffu, q.s, o), __shfl_xor_sync(0xffffffffu, q.c, o)};
+    p = merge(p, a);
+    q = merge(q, b);
   }
-  return p;
 }
 
 // Chunk partials climb the set's radix-32 tree: the block that completes the
@@ -795,16 +800,22 @@ __device__ void climb_tree(const Program& P, const Pass& pass, S& sm, int set, i
     if (!sm.last) return;
     __threadfence();
     const int64_t c0 = base + lvl + first;
-    for (int q = warp; q < Q; q += kWarps) {
-      Pair p{0.0, 0.0};
+    for (int q = warp; q < Q; q += 2 * kWarps) {  // two quantities at a time
+      const int q2 = q + kWarps;
+      Pair p{0.0, 0.0}, r{0.0, 0.0};
       if (lane < m) {
-        p.s = __ldcg(pass.tree + (c0 + lane) * 2 * Q + q);
-        p.c = __ldcg(pass.tree + (c0 + lane) * 2 * Q + Q + q);
+        const double* row = pass.tree + (c0 + lane) * 2 * Q;
+        p = {__ldcg(row + q), __ldcg(row + Q + q)};
+        if (q2 < Q) r = {__ldcg(row + q2), __ldcg(row + Q + q2)};
       }
-      p = warp_merge(p);
+      warp_merge2(p, r, m);
       if (lane == 0) {
         pass.tree[pnode * 2 * Q + q] = p.s;
         pass.tree[pnode * 2 * Q + Q + q] = p.c;
+        if (q2 < Q) {
+          pass.tree[pnode * 2 * Q + q2] = r.s;
+          pass.tree[pnode * 2 * Q + Q + q2] = r.c;
+        }
       }
     }
     if (warp == 0) {
@@ -834,22 +845,23 @@ __device__ void climb_tree(const Program& P, const Pass& pass, S& sm, int set, i
       pr[2 + 2 * k] = g.s;
       pr[3 + 2 * k] = g.c;
     }
-  } else if (tid == 0) {
-    const int flag = pass.flags[set] + __ldcg(pass.tree_bad + root);
-    pass.flags[set] = flag;
+  } else if (tid <= P.n_free && !pass.pairs) {
+    // thread 0: the NLL; thread 1 + k: free parameter k
+    const double* row = pass.tree + root * 2 * Q;
     double* o = pass.out + (size_t)set * (1 + P.n_free);
-    const double s0 = __ldcg(pass.tree + root * 2 * Q) + __ldcg(pass.tree + root * 2 * Q + Q);
     double ext = 0.0, dext = 0.0;
     if (P.ext) extended_term(P, pass, set, (double)n_events, &ext, &dext);
-    o[0] = flag ? INFINITY : ext - s0;
-    if (pass.want_grad) {
-      for (int k = 0; k < P.n_free; ++k) {
-        double gk = 0.0;
-        for (int sl = 0; sl < P.n_slots; ++sl)
-          if (P.slot_free[sl] == k)
-            gk += __ldcg(pass.tree + root * 2 * Q + 1 + sl) + __ldcg(pass.tree + root * 2 * Q + Q + 1 + sl);
-        o[1 + k] = (k == P.ext_free ? dext : 0.0) - gk;
-      }
+    if (tid == 0) {
+      const int flag = pass.flags[set] + __ldcg(pass.tree_bad + root);
+      pass.flags[set] = flag;
+      const double s0 = __ldcg(row) + __ldcg(row + Q);
+      o[0] = flag ? INFINITY : ext - s0;
+    } else if (pass.want_grad) {
+      const int k = tid - 1;
+      double gk = 0.0;
+      for (int sl = 0; sl < P.n_slots; ++sl)
+        if (P.slot_free[sl] == k) gk += __ldcg(row + 1 + sl) + __ldcg(row + Q + 1 + sl);
+      o[1 + k] = (k == P.ext_free ? dext : 0.0) - gk;
     }
   }
 }
@@ -1040,15 +1052,18 @@ __global__ void __launch_bounds__(kLanes, ff_min_blocks(kShape)) events_ff(const
   const int n_units = n_items * parts;
   int kc_set = -1, c_set = -1;  // sets whose constants the block holds (block-uniform)
   pdl_wait();  // K1 has reset the counter and written the constants
-  // One unit of lookahead: thread 0 claims the next unit while the block
-  // works on the current one, so the claim's round trip is hidden.
+  // Thread 0 claims the next unit when the fast pass over the current one is
+  // done, so the claim's round trip is hidden by the rest of the unit.  (Not
+  // at the unit's start: a block would hold two units from its first moment,
+  // and with fewer than two units per block half of the blocks would idle
+  // beside them.  Decay model, 1064 units for 1064 blocks: 133 us so, 84 now;
+  // 1e6 events 60 and 43 us.)
   int next_u = tid == 0 ? atomicAdd(pass.counter, 1) : 0;
   while (true) {
     if (tid == 0) sm.item = next_u;
     __syncthreads();
     const int u = sm.item;
     if (u >= n_units) break;
-    if (tid == 0) next_u = atomicAdd(pass.counter, 1);
     const int it = u / parts, part = u % parts;
     const int set = pass.items[it].x, chunk = pass.items[it].y;
     const int64_t s_begin = pass.offsets[set], s_end = pass.offsets[set + 1];
@@ -1070,7 +1085,7 @@ __global__ void __launch_bounds__(kLanes, ff_min_blocks(kShape)) events_ff(const
     // next event's observables are loaded one iteration ahead
     const int rem = (int)(s_end - base < (int64_t)kChunk ? s_end - base : (int64_t)kChunk);
     int off = tid + k0 * kLanes;
-    FFRaw<kShape> nxt;
+    FFRaw<kShape> nxt{};  // (a lane without events converts it too)
     if (off < rem) nxt = ff_load_raw<kShape, kF32>(cols, col, base + off);
 #pragma unroll 1
     for (int k = k0; k < k0 + kPartK; ++k, off += kLanes) {
@@ -1082,6 +1097,7 @@ __global__ void __launch_bounds__(kLanes, ff_min_blocks(kShape)) events_ff(const
       myslow |= (st == 1 ? 1u : 0u) << k;
       myfb |= (st == 2 ? 1u : 0u) << k;
     }
+    if (tid == 0) next_u = atomicAdd(pass.counter, 1);
     if constexpr (kShape == SHAPE_PROD3 && kGrad) {
       // moment 13: the lane's events summed in float-float (those present
       // in its part, less the ones the FP64 path takes whole)
