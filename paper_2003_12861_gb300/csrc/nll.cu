@@ -607,7 +607,7 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
       }
       case EXPR: {
         double f;
-        if constexpr (kExpr) v[n] = expr_eval(P, q, c + 1 + q.n_par, x[q.col], 0, &f, nullptr) ? f * c[0] : NAN;
+        if constexpr (kExpr) v[n] = expr_eval<false>(P, q, c + 1 + q.n_par, x[q.col], &f, nullptr) == 0 ? f * c[0] : NAN;
         break;
       }
       case SUM: {
@@ -663,7 +663,7 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
       case EXPR: {  // dv/dp_j = (df/dp_j - f dlogI/dp_j) / I, with no division by f (which may underflow)
         if constexpr (kExpr) {
           double f, df[kMaxPar];
-          expr_eval(P, q, c + 1 + q.n_par, x[q.col], q.n_par, &f, df);
+          expr_eval<true>(P, q, c + 1 + q.n_par, x[q.col], &f, df);
           const double w = a * c[0];
           for (int j = 0; j < q.n_par; ++j) g[s0 + j] += w * (df[j] - f * c[1 + j]);
         }

@@ -108,7 +108,7 @@ __device__ __noinline__ double factor_value(const Program& P, const double* __re
       }
       case EXPR: {
         double f;
-        v[n] = expr_eval(P, q, c + 1 + q.n_par, xc, 0, &f, nullptr) ? f * c[0] : NAN;
+        v[n] = expr_eval<false>(P, q, c + 1 + q.n_par, xc, &f, nullptr) == 0 ? f * c[0] : NAN;
         break;
       }
       case SUM: {
