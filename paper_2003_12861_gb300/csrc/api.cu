@@ -126,8 +126,9 @@ bool ensure_workspace(const rf_model* m, rf_data* d) {
   Workspace& w = d->ws;
   const Program& P = m->m.prog;
   const int Q = 1 + P.n_slots;
+  const int gen_parts = parts_for(d->total_chunks, SHAPE_GENERIC);
   if (w.ready && w.n_const == P.n_const && w.n_free == P.n_free && w.Q == Q &&
-      (m->m.shape == SHAPE_GENERIC || w.ffc.p))
+      (m->m.shape == SHAPE_GENERIC ? gen_parts == 1 || w.gen_part.p : w.ffc.p != nullptr))
     return true;
   const size_t S = d->n_sets;
   const size_t nodes = (size_t)std::max<int64_t>(1, d->total_nodes);
@@ -140,6 +141,9 @@ bool ensure_workspace(const rf_model* m, rf_data* d) {
             w.counter.ensure(sizeof(int32_t)) && w.slow.ensure(sizeof(unsigned long long)) &&
             w.slot_counter.ensure(sizeof(int32_t) * kPassSlots) &&
             w.slot_slow.ensure(sizeof(unsigned long long) * kPassSlots) &&
+            (m->m.shape != SHAPE_GENERIC || gen_parts == 1 ||
+             (w.gen_part.ensure(sizeof(double) * nodes * gen_parts * 2 * Q) &&
+              w.gen_info.ensure(sizeof(int32_t) * nodes * gen_parts))) &&
             (m->m.shape == SHAPE_GENERIC ||
              (w.ffc.ensure(sizeof(float) * S * kFFConst) &&
               w.part_m.ensure(sizeof(float) * nodes * kMaxParts * kPartFloats) &&
@@ -187,8 +191,8 @@ Pass make_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* d_
   p.ff_shape = m->m.shape;
   p.ffc = m->m.shape == SHAPE_GENERIC ? nullptr : (float*)w.ffc.p;
   p.part_m = (float*)w.part_m.p;
-  p.part_fb = (double*)w.part_fb.p;
-  p.part_info = (int32_t*)w.part_info.p;
+  p.part_fb = (double*)(m->m.shape == SHAPE_GENERIC ? w.gen_part.p : w.part_fb.p);
+  p.part_info = (int32_t*)(m->m.shape == SHAPE_GENERIC ? w.gen_info.p : w.part_info.p);
   p.parts = parts_for(d->total_chunks, m->m.shape);
   p.pairs = nullptr;
   return p;

@@ -51,6 +51,7 @@ struct Workspace {
   bool ready = false;
   int n_const = -1, n_free = -1, Q = -1;
   DevBuf consts, theta, out, flags, tree, tree_bad, tickets, counter, slow, ffc, part_m, part_fb, part_info;
+  DevBuf gen_part, gen_info;  // part records of the generic kernel
   // work and slow-event counters of passes that may run concurrently on
   // other streams (launch_pass with slot >= 0)
   DevBuf slot_counter, slot_slow;

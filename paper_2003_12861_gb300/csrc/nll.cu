@@ -26,7 +26,6 @@ constexpr double kSqrt1_2 = 0.70710678118654752440;
 constexpr double kSqrt2Pi = 2.50662827463100050242;
 constexpr double kInvSqrt2Pi = 0.39894228040143267794;
 constexpr double kInvSqrtPi = 0.56418958354775628695;
-constexpr double kTwoInvSqrtPi = 1.12837916709551257390;
 // Below this z the erfc factor of the decay-resolution convolution equals 2
 // to better than 1e-22 relative and its derivative term is below 1e-21 of
 // the exponential's, so the event takes the one-exponential fast path.
@@ -541,6 +540,18 @@ __device__ __forceinline__ double logprod64_log(const LogProd64& L) {
   return log(L.m) + (double)L.e * 0.69314718055994530942;
 }
 
+// p > 0 and finite, and z >= kSlowZ (or NaN), by the bits: an FP64 comparison
+// would take the FP64 unit like any other FP64 instruction.
+__device__ __forceinline__ bool positive_finite(double p) {
+  return (unsigned)__double2hiint(p) < 0x7ff00000u && (__double2hiint(p) | __double2loint(p)) != 0;
+}
+__device__ __forceinline__ bool is_slow_z(double z) {
+  constexpr unsigned hi = 0xc01c0000u;  // -7
+  const unsigned h = (unsigned)__double2hiint(z);
+  return h < hi || (h == hi && __double2loint(z) == 0);
+}
+static_assert(kSlowZ == -7.0, "is_slow_z holds its bits");
+
 // Generic graph interpreter for one event.  kFull = false: the fast path,
 // which returns false (and adds nothing) when some node needs its slow path.
 // Multiplies p into the lane's running product L (the log p term) and adds
@@ -550,10 +561,21 @@ __device__ __forceinline__ double logprod64_log(const LogProd64& L) {
 // one factor's sub-program (a PROD factor's nodes are contiguous in program
 // order and refer only to each other), whose log p and slot gradients are
 // then those of that factor alone.
-template <bool kFull, bool kGrad, bool kExpr = false>
+// Only FP64 operations count here (64 cycles of the unit each; everything
+// else hides behind them), so what the value pass has computed (u, the
+// unnormalised value, a program's derivatives) is kept for the gradient pass
+// in per-thread memory, and no node divides by what it multiplied with
+// (kKept; the float-float kernels' rare events compute it again, as those
+// arrays would cost their event loop 1 % of its time).
+template <bool kFull, bool kGrad, bool kExpr = false, bool kKept = true>
 __device__ bool eval_generic(const Program& P, const double* __restrict__ C, const double* x, double* acc,
                              LogProd64& L, int* bad, int n0 = 0, int n1 = -1) {
   double v[kMaxPdf];
+  constexpr bool kKeep = kGrad && kKept;
+  double w1[kKeep ? kMaxPdf : 1];             // per node: u, or the unnormalised value
+  double w2[kKeep && kFull ? kMaxPdf : 1];    // GAUSSEXP: exp(-u^2/2)
+  double f1[kKeep && kFull ? kMaxPdf : 1];    // and the convolution
+  double dex[kGrad && kExpr ? kMaxSlots : 1]; // EXPR: derivatives by slot
   const int N = n1 < 0 ? P.n_pdf : n1;
   for (int n = n0; n < N; ++n) {
     const PNode& q = P.node[n];
@@ -561,6 +583,7 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
     switch (q.kind) {
       case GAUSS: {
         const double u = (x[q.col] - c[0]) * c[1];
+        if constexpr (kKeep) w1[n] = u;
         v[n] = exp(-0.5 * u * u) * c[2];
         break;
       }
@@ -568,14 +591,19 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
       case GAUSSEXP: {
         const double u = (x[q.col] - c[0]) * c[1], s = c[2];
         const double z = (s - u) * kSqrt1_2;
+        if constexpr (kKeep) w1[n] = u;
         double f;
-        if (!kFull) {
-          if (z >= kSlowZ) return false;
+        if constexpr (!kFull) {
+          if (is_slow_z(z)) return false;
           f = exp(s * (0.5 * s - u));
-        } else if (z > 0.0) {
-          f = 0.5 * exp(-0.5 * u * u) * erfcx(z);
         } else {
-          f = 0.5 * exp(s * (0.5 * s - u)) * erfc(z);
+          const bool right = z > 0.0;
+          const double g = kGrad || right ? exp(-0.5 * u * u) : 0.0;
+          f = right ? 0.5 * g * erfcx(z) : 0.5 * exp(s * (0.5 * s - u)) * erfc(z);
+          if constexpr (kKeep) {
+            w2[n] = g;
+            f1[n] = f;
+          }
         }
         v[n] = f * c[4];
         break;
@@ -586,9 +614,12 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
         double t0 = 1.0, t1 = xp, sh = 1.0;
         for (int k = 1; k <= np; ++k) {
           sh += c[3 + np + k - 1] * t1;
-          const double t2 = 2.0 * xp * t1 - t0;
-          t0 = t1; t1 = t2;
+          if (k < np) {
+            const double t2 = 2.0 * xp * t1 - t0;
+            t0 = t1; t1 = t2;
+          }
         }
+        if constexpr (kKeep) w1[n] = sh;
         v[n] = sh * c[2];
         break;
       }
@@ -597,7 +628,9 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
         const double xv = x[q.col];
         double sh = 0.0;
         for (int k = np; k >= 1; --k) sh = (sh + c[1 + np + k - 1]) * xv;
-        v[n] = (1.0 + sh) * c[0];
+        sh += 1.0;
+        if constexpr (kKeep) w1[n] = sh;
+        v[n] = sh * c[0];
         break;
       }
       case POISSON: {
@@ -606,8 +639,11 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
         break;
       }
       case EXPR: {
-        double f;
-        if constexpr (kExpr) v[n] = expr_eval<false>(P, q, c + 1 + q.n_par, x[q.col], &f, nullptr) == 0 ? f * c[0] : NAN;
+        if constexpr (kExpr) {
+          double f;
+          v[n] = expr_eval<kGrad>(P, q, c + 1 + q.n_par, x[q.col], &f, dex + (kGrad ? q.slot0 : 0)) != 1 ? f * c[0] : NAN;
+          if constexpr (kGrad) w1[n] = f;
+        }
         break;
       }
       case SUM: {
@@ -617,8 +653,8 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
         break;
       }
       case PROD: {
-        double r = 1.0;
-        for (int j = 0; j < q.n_child; ++j) r *= v[q.child[j]];
+        double r = v[q.child[0]];
+        for (int j = 1; j < q.n_child; ++j) r *= v[q.child[j]];
         v[n] = r;
         break;
       }
@@ -626,7 +662,7 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
     }
   }
   const double p = v[N - 1];
-  if (!(p > 0.0) || !isfinite(p)) {
+  if (!positive_finite(p)) {
     ++*bad;
     return true;
   }
@@ -645,10 +681,9 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
     const int s0 = q.slot0;
     switch (q.kind) {
       case GAUSS: {
-        const double w = a * v[n];
-        const double u = (x[q.col] - c[0]) * c[1];
-        g[s0] += w * (u * c[1] - c[3]);
-        g[s0 + 1] += w * (u * u * c[1] - c[4]);
+        const double w = a * v[n], u = kKeep ? w1[n] : (x[q.col] - c[0]) * c[1], ui = u * c[1];
+        g[s0] += w * (ui - c[3]);
+        g[s0 + 1] += w * (u * ui - c[4]);
         break;
       }
       case EXPO: {
@@ -662,51 +697,51 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
       }
       case EXPR: {  // dv/dp_j = (df/dp_j - f dlogI/dp_j) / I, with no division by f (which may underflow)
         if constexpr (kExpr) {
-          double f, df[kMaxPar];
-          expr_eval<true>(P, q, c + 1 + q.n_par, x[q.col], &f, df);
-          const double w = a * c[0];
-          for (int j = 0; j < q.n_par; ++j) g[s0 + j] += w * (df[j] - f * c[1 + j]);
+          const double w = a * c[0], f = w1[n];
+          for (int j = 0; j < q.n_par; ++j) g[s0 + j] += w * (dex[s0 + j] - f * c[1 + j]);
         }
         break;
       }
       case GAUSSEXP: {
-        const double w = a * v[n];
-        const double u = (x[q.col] - c[0]) * c[1], s = c[2], it = c[3];
-        double dt = s * (u - s) * it, dm = it, ds = s * it;
-        if (kFull) {
-          const double z = (s - u) * kSqrt1_2;
-          const double R = kTwoInvSqrtPi / erfcx(z);  // exp(-z^2)/erfc(z) * 2/sqrt(pi)
-          dt -= R * (-s * it * kSqrt1_2);
-          dm -= R * (c[1] * kSqrt1_2);
-          ds -= R * ((it + u * c[1]) * kSqrt1_2);
+        const double u = kKeep ? w1[n] : (x[q.col] - c[0]) * c[1], s = c[2], it = c[3], sit = s * it;
+        if constexpr (!kFull) {
+          const double w = a * v[n];
+          g[s0] += w * (sit * (u - s) - c[5]);
+          g[s0 + 1] += w * (it - c[6]);
+          g[s0 + 2] += w * (sit - c[7]);
+        } else {  // df = f dA - exp(-u^2/2)/sqrt(pi) dz, with no division by f
+          const double w = a * c[4], f = kKeep ? f1[n] : v[n] / c[4];
+          const double h = (kKeep ? w2[n] : exp(-0.5 * u * u)) * kInvSqrt2Pi;
+          g[s0] += w * (f * (sit * (u - s) - c[5]) + h * sit);
+          g[s0 + 1] += w * (f * (it - c[6]) - h * c[1]);
+          g[s0 + 2] += w * (f * (sit - c[7]) - h * (it + u * c[1]));
         }
-        g[s0] += w * (dt - c[5]);
-        g[s0 + 1] += w * (dm - c[6]);
-        g[s0 + 2] += w * (ds - c[7]);
         break;
       }
       case CHEB: {
         const int np = q.n_par;
         const double xp = x[q.col] * c[0] - c[1];
-        const double sh = v[n] / c[2];
+        const double sh = kKeep ? w1[n] : v[n] / c[2];
         const double ai = a * c[2];
         double t0 = 1.0, t1 = xp;
         for (int k = 1; k <= np; ++k) {
           g[s0 + k - 1] += ai * (t1 - sh * c[3 + k - 1]);
-          const double t2 = 2.0 * xp * t1 - t0;
-          t0 = t1; t1 = t2;
+          if (k < np) {
+            const double t2 = 2.0 * xp * t1 - t0;
+            t0 = t1; t1 = t2;
+          }
         }
         break;
       }
       case POLY: {
         const int np = q.n_par;
         const double xv = x[q.col];
-        const double sh = v[n] / c[0];
+        const double sh = kKeep ? w1[n] : v[n] / c[0];
         const double ai = a * c[0];
-        double xk = 1.0;
+        double xk = xv;
         for (int k = 1; k <= np; ++k) {
-          xk *= xv;
           g[s0 + k - 1] += ai * (xk - sh * c[1 + k - 1]);
+          if (k < np) xk *= xv;
         }
         break;
       }
@@ -721,9 +756,11 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
         const int nc = q.n_child;
         for (int j = 0; j < nc; ++j) {
           double o = a;
-          for (int i = 0; i < nc; ++i)
+          const int last = j == nc - 1 ? nc - 2 : nc - 1;  // the last factor but j
+          for (int i = 0; i < last; ++i)
             if (i != j) o *= v[q.child[i]];
-          ad[q.child[j]] += o;
+          if (last >= 0) ad[q.child[j]] += o * v[q.child[last]];
+          else ad[q.child[j]] += o;
         }
         break;
       }
@@ -742,7 +779,7 @@ struct SmemT {
   double C[kMaxConst];
   double wsum[kWarps][kQMax];
   int wbad[kWarps];
-  QT queue[kWarps][kQueue];
+  alignas(8) QT queue[kWarps][kQueue];
   int qn[kWarps];
   int item;
   int last;
@@ -882,61 +919,121 @@ __device__ void write_chunk(const Program& P, const Pass& pass, S& sm, int bad, 
   climb_tree(P, pass, sm, set, chunk, n_events);
 }
 
-// Writes the chunk's partial (warp sums merged in a fixed order) to its
-// level-0 tree node and climbs the tree.
-__device__ void finish_chunk(const Program& P, const Pass& pass, Smem& sm, double* acc, int bad, int set,
-                             int chunk, int64_t n_events) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int Q = pass.Q;
-  for (int q = 0; q < Q; ++q) {
-    const double w = warp_sum(acc[q]);
-    if (lane == 0) sm.wsum[warp][q] = w;
+// Sums acc[0..Q) over the lanes of a warp into out[0..Q), eight quantities at
+// a time: the lanes' values go to shared memory (buf: 256 doubles of the
+// warp, a quantity's row rotated by its index so that neither side meets a
+// bank conflict), four lanes per quantity add eight lanes' values each and
+// two butterfly levels join them: 9 FP64 additions for eight quantities
+// where butterflies take 40.
+__device__ __forceinline__ void warp_sums(const double* acc, int Q, double* buf, double* out, int lane) {
+  const int j = lane >> 2, r = lane & 3;
+  for (int q0 = 0; q0 < Q; q0 += 8) {
+    const int m = min(8, Q - q0);
+    for (int k = 0; k < m; ++k) buf[k * 32 + ((lane + k) & 31)] = acc[q0 + k];
+    __syncwarp();
+    double x = 0.0;
+    if (j < m) {
+      x = buf[j * 32 + ((r * 8 + j) & 31)];
+#pragma unroll
+      for (int i = 1; i < 8; ++i) x += buf[j * 32 + ((r * 8 + i + j) & 31)];
+    }
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    if (j < m && r == 0) out[q0 + j] = x;
+    __syncwarp();
   }
+}
+
+// Ends a work unit: the block's sums (lanes, then warps in a fixed order) go
+// to the chunk's level-0 tree node if the unit is the whole chunk, otherwise
+// to the part's record; the block that completes the chunk's last part
+// merges the parts in part order.  Then the climb up the tree.
+__device__ void finish_unit(const Program& P, const Pass& pass, Smem& sm, const double* acc, int bad, int set,
+                            int chunk, int part, int64_t n_events) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int Q = pass.Q, parts = pass.parts;
+  warp_sums(acc, Q, (double*)sm.queue[warp], sm.wsum[warp], lane);
   bad = warp_sum_int(bad);
   if (lane == 0) sm.wbad[warp] = bad;
   __syncthreads();
   const int64_t node = pass.tree_base[set] + chunk;
+  const int64_t rec = node * parts + part;
+  double* dst = parts == 1 ? pass.tree + node * 2 * Q : pass.part_fb + rec * 2 * Q;
   if (tid < Q) {
     Pair a = merge({sm.wsum[0][tid], 0.0}, {sm.wsum[1][tid], 0.0});
     Pair b = merge({sm.wsum[2][tid], 0.0}, {sm.wsum[3][tid], 0.0});
     Pair r = merge(a, b);
-    pass.tree[node * 2 * Q + tid] = r.s;
-    pass.tree[node * 2 * Q + Q + tid] = r.c;
+    dst[tid] = r.s;
+    dst[Q + tid] = r.c;
   }
-  if (tid == 0) pass.tree_bad[node] = sm.wbad[0] + sm.wbad[1] + sm.wbad[2] + sm.wbad[3];
+  if (tid == 0)
+    *(parts == 1 ? pass.tree_bad + node : pass.part_info + rec) = sm.wbad[0] + sm.wbad[1] + sm.wbad[2] + sm.wbad[3];
+  if (parts > 1) {
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+      const int t = atomicAdd(&pass.tickets[node], 1);
+      sm.last = (t == parts - 1);
+      if (sm.last) pass.tickets[node] = 0;
+    }
+    __syncthreads();
+    if (!sm.last) return;
+    __threadfence();
+    if (tid < Q) {
+      const double* p = pass.part_fb + node * parts * 2 * Q + tid;
+      Pair r{__ldcg(p), __ldcg(p + Q)};
+      for (int i = 1; i < parts; ++i) r = merge(r, {__ldcg(p + i * 2 * Q), __ldcg(p + i * 2 * Q + Q)});
+      pass.tree[node * 2 * Q + tid] = r.s;
+      pass.tree[node * 2 * Q + Q + tid] = r.c;
+    }
+    if (tid == 0) {
+      int b = 0;
+      for (int i = 0; i < parts; ++i) b += __ldcg(pass.part_info + node * parts + i);
+      pass.tree_bad[node] = b;
+    }
+  }
   climb_tree(P, pass, sm, set, chunk, n_events);
 }
 
-// Generic fused event kernel: persistent blocks of 128 threads take 4096-event
-// chunks from the work counter; lane l evaluates events l, l+128, ... of the
-// chunk in order.  Events that need a node's slow path are queued per warp
+// Generic fused event kernel: persistent blocks of 128 threads take units (a
+// 4096-event chunk or one of its pass.parts parts) from the work counter;
+// lane l evaluates events l, l+128, ... of the unit in order.  Events that
+// need a node's slow path are queued per warp
 // (ballot order) and evaluated after the fast pass, so the warp stays
 // converged; the lane order of additions is still fixed by the data alone.
+// The next unit is claimed after the unit's events, when the other blocks
+// have had their share.
+// Bound by the FP64 unit (84 % busy, 91 FP64 instructions an event for the
+// decay model).  Before / after the split into parts, one evaluation of a
+// program per event and the values kept for the gradient pass: decay model
+// 1e4 events 203 -> 41 us, 1e6 285 -> 217, 4e6 862 -> 705; program model 1e4
+// 629 -> 54, 1e6 822 -> 355.
 template <bool kGrad, bool kExpr>
 __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__ Program P,
                                                          const __grid_constant__ Columns cols, Pass pass) {
   __shared__ Smem sm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int Q = kGrad ? 1 + P.n_slots : 1;
-  const int n_items = pass.dyn ? pass.dyn[1] : pass.n_items;
-  if (n_items == 0) return;
+  const int n_units = (pass.dyn ? pass.dyn[1] : pass.n_items) * pass.parts;
+  if (n_units == 0) return;
   pdl_wait();
+  const int per_lane = kPerLane / pass.parts;
+  if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
+  __syncthreads();
   while (true) {
-    if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
-    __syncthreads();
-    const int it = sm.item;
-    if (it >= n_items) break;
+    const int u = sm.item;
+    if (u >= n_units) break;
+    const int it = u / pass.parts, part = u % pass.parts;
     const int set = pass.items[it].x, chunk = pass.items[it].y;
     const int64_t s_begin = pass.offsets[set], s_end = pass.offsets[set + 1];
-    const int64_t base = s_begin + (int64_t)chunk * kChunk;
+    const int64_t base = s_begin + (int64_t)chunk * kChunk + part * (per_lane * kLanes);
     for (int i = tid; i < P.n_const; i += kLanes) sm.C[i] = pass.consts[(size_t)set * P.n_const + i];
     __syncthreads();
     double acc[kQMax];
-    for (int q = 0; q < kQMax; ++q) acc[q] = 0.0;
+    for (int q = 0; q < pass.Q; ++q) acc[q] = 0.0;
     int bad = 0, qcnt = 0;
     LogProd64 L = logprod64_init();
     double x[kMaxObs];
-    for (int k = 0; k < kPerLane; ++k) {
+    for (int k = 0; k < per_lane; ++k) {
       const int64_t e = base + tid + (int64_t)k * kLanes;
       bool slow = false;
       if (e < s_end) {
@@ -956,9 +1053,10 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
       for (int c = 0; c < P.n_obs; ++c) x[c] = load_col(cols, c, e);
       eval_generic<true, kGrad, kExpr>(P, sm.C, x, acc, L, &bad);
     }
+    if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
     acc[0] += logprod64_log(L);
-    (void)Q;
-    finish_chunk(P, pass, sm, acc, bad, set, chunk, s_end - s_begin);
+    __syncwarp();
+    finish_unit(P, pass, sm, acc, bad, set, chunk, part, s_end - s_begin);
     __syncthreads();
   }
 }
@@ -1152,14 +1250,14 @@ __global__ void __launch_bounds__(kLanes, ff_min_blocks(kShape)) events_ff(const
         myfb &= myfb - 1u;
         const int64_t e = base + tid + (int64_t)k * kLanes;
         for (int c = 0; c < P.n_obs; ++c) x[c] = load_col(cols, c, e);
-        eval_generic<true, kGrad>(P, sm.C, x, acc64, L64, &bad);
+        eval_generic<true, kGrad, false, false>(P, sm.C, x, acc64, L64, &bad);
       }
       while (myfb_f) {  // PROD3: the decay factor's sub-program, program nodes 3..5
         const int k = __ffs(myfb_f) - 1;
         myfb_f &= myfb_f - 1u;
         const int64_t e = base + tid + (int64_t)k * kLanes;
         for (int c = 0; c < P.n_obs; ++c) x[c] = load_col(cols, c, e);
-        eval_generic<true, kGrad>(P, sm.C, x, acc64, L64, &bad, 3, 6);
+        eval_generic<true, kGrad, false, false>(P, sm.C, x, acc64, L64, &bad, 3, 6);
       }
       acc64[0] += logprod64_log(L64);
     }
@@ -1323,7 +1421,7 @@ void launch_events(const Program& P, Shape shape, const Columns& cols, const Pas
   const int bps = blocks_per_sm > 0 ? blocks_per_sm : 8;
   int grid = n_sm * bps;
   const Shape sh = (pass.ff_shape != SHAPE_GENERIC && pass.ffc) ? shape : SHAPE_GENERIC;
-  const int64_t units = sh == SHAPE_GENERIC ? (int64_t)pass.n_items : (int64_t)pass.n_items * pass.parts;
+  const int64_t units = (int64_t)pass.n_items * pass.parts;
   if (grid > units) grid = (int)units;
   note_launches(1, st);
   timing_begin(st);

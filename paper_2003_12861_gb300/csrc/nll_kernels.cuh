@@ -38,10 +38,12 @@ struct Pass {
   float* ffc;               // n_sets x 512 floats of its parameter-point constants, or null
   // Float-float kernels: per chunk, `parts` part records (indexed by the
   // chunk's level-0 tree node x parts + part; room for kMaxParts).
-  int32_t parts;            // work units per chunk (1 or 4), fixed per dataset
+  int32_t parts;            // work units per chunk (parts_for), fixed per dataset
   float* part_m;            // 32 floats per part: its moment sums (float-float pairs)
   double* part_fb;          // Q doubles per part: its FP64 fallback sums (valid if info bit 0)
   int32_t* part_info;       // per part: bit 0 = fallback sums present, bits 1.. = bad events
+  // Generic kernel with parts > 1: part_fb holds 2 Q doubles per part (sums,
+  // compensations), part_info its bad events.
   // Partial mode (null otherwise): per set (1 + n_free) (sum, compensation)
   // pairs of (sum log p, d/dtheta_k sum log p), not negated, for a later
   // ordered combine across shards; out is not written.
@@ -70,9 +72,23 @@ __host__ __device__ constexpr int ff_min_blocks(int shape) { return shape == SHA
 // is a function of the dataset's chunk count and the model's kernel only,
 // never of the launch: a dataset's results do not depend on how it is
 // launched.
-constexpr int kMaxParts = 4;
-constexpr int kRefSMs = 152;
+//
+// The generic kernel's events are bound by the FP64 unit (1 us a warp), and
+// per unit it pays a pass over the queued events, a logarithm and the sums.
+// It splits chunks, up to 16 ways, until there are six units for each SM:
+// us with 1 | 2 | 4 | 8 | 16 parts for the decay model with the 8-block grid,
+// 1e4 events 181 | 100 | 69 | 47 | 41, 3e5 193 | 115 | 89 | 91 | 125, 1e6
+// 244 | 226 | 217 | 243 | 351, 4e6 705 | 681 | 760 | 908 | 1269; for the
+// program model 1e4 483 | 252 | 137 | 81 | 54, 1e6 597 | 416 | 355 | 347 |
+// 396, 4e6 1300 | 1250 | 1314 | 1289 | 1381.
+constexpr int kMaxParts = 4, kMaxPartsGeneric = 16;
+constexpr int kRefSMs = 152, kGenericUnits = kRefSMs * 6;
 inline int parts_for(int64_t total_chunks, int shape) {
+  if (shape == SHAPE_GENERIC) {
+    int P = 1;
+    while (P < kMaxPartsGeneric && total_chunks * P < kGenericUnits) P *= 2;
+    return P;
+  }
   const int64_t wave = (int64_t)kRefSMs * ff_min_blocks(shape);
   int P = 1;
   while (P < kMaxParts && total_chunks * P < wave) P *= 2;

@@ -44,7 +44,8 @@ struct Layout {
 
 // Header (first 256 bytes): int32 counter @0, u64 slow-event count @8,
 // int64 offsets[2] @16, int64 tree base @32, int32 active set @40.
-Layout layout_for(int64_t chunks, int64_t nodes, int n_const, int Q, bool parts, int shape) {
+Layout layout_for(int64_t chunks, int64_t nodes, int n_const, int Q, int shape) {
+  const bool ff = shape != SHAPE_GENERIC;
   const size_t np = (size_t)parts_for(chunks, shape);
   Layout L{};
   L.consts = 256;
@@ -53,11 +54,12 @@ Layout layout_for(int64_t chunks, int64_t nodes, int n_const, int Q, bool parts,
   L.bad = L.items + up256(sizeof(int2) * (size_t)(chunks > 0 ? chunks : 1));
   L.tickets = L.bad + up256(sizeof(int32_t) * (size_t)(nodes > 0 ? nodes : 1));
   L.tree = L.tickets + up256(sizeof(int32_t) * (size_t)(nodes > 0 ? nodes : 1));
-  // float-float kernels only: the part records of every chunk
-  const size_t nn = parts ? (size_t)(nodes > 0 ? nodes : 1) : 0;
+  // the part records of every chunk (the generic kernel's only when it splits
+  // chunks, two doubles a quantity)
+  const size_t nn = ff || np > 1 ? (size_t)(nodes > 0 ? nodes : 1) : 0;
   L.part_m = L.tree + up256(sizeof(double) * 2 * (size_t)Q * (size_t)(nodes > 0 ? nodes : 1));
-  L.part_fb = L.part_m + up256(sizeof(float) * np * kPartFloats * nn);
-  L.part_info = L.part_fb + up256(sizeof(double) * np * (size_t)Q * nn);
+  L.part_fb = L.part_m + up256(ff ? sizeof(float) * np * kPartFloats * nn : 0);
+  L.part_info = L.part_fb + up256(sizeof(double) * np * (size_t)Q * nn * (ff ? 1 : 2));
   L.total = L.part_info + sizeof(int32_t) * np * nn;
   return L;
 }
@@ -87,7 +89,7 @@ __global__ void noalloc_setup(unsigned char* base, Layout L, int64_t n_events, i
 size_t scratch_bytes(const rf_model* m, int64_t n_events) {
   const Program& P = m->m.prog;
   const int64_t chunks = (n_events + kChunk - 1) / kChunk;
-  return layout_for(chunks, tree_nodes(chunks), P.n_const, 1 + P.n_slots, m->m.shape != SHAPE_GENERIC, m->m.shape).total;
+  return layout_for(chunks, tree_nodes(chunks), P.n_const, 1 + P.n_slots, m->m.shape).total;
 }
 
 }  // namespace
@@ -125,7 +127,7 @@ extern "C" rf_status rf_nll_grad_noalloc(const rf_model* m, const void* const* d
   const int64_t chunks = (n_events + kChunk - 1) / kChunk;
   const int64_t nodes = tree_nodes(chunks);
   const int Q = 1 + P.n_slots;
-  const Layout L = layout_for(chunks, nodes, P.n_const, Q, m->m.shape != SHAPE_GENERIC, m->m.shape);
+  const Layout L = layout_for(chunks, nodes, P.n_const, Q, m->m.shape);
   if (L.total > kScratchBytes || chunks > (int64_t)0x7fffffff) {
     const double per_chunk = (double)L.total / (double)(chunks > 0 ? chunks : 1);
     char msg[256];
