@@ -208,9 +208,15 @@ Columns make_columns(const rf_data* d) {
 }
 
 bool launch_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* d_theta, double* d_out,
-                 int32_t* d_flags, bool grad, cudaStream_t st, int slot, const int32_t* dyn) {
+                 int32_t* d_flags, bool grad, cudaStream_t st, int slot, const int32_t* dyn, int32_t* flags_out,
+                 const double* theta1) {
   Pass pass = make_pass(m, d, plan, d_theta, d_out, d_flags, grad);
   pass.dyn = dyn;
+  pass.flags_out = flags_out;
+  if (theta1) {
+    pass.n_theta1 = m->m.prog.n_free;
+    std::memcpy(pass.theta1, theta1, sizeof(double) * m->m.prog.n_free);
+  }
   if (slot >= 0 && slot < kPassSlots) {
     pass.counter = (int32_t*)d->ws.slot_counter.p + slot;
     pass.slow = (unsigned long long*)d->ws.slot_slow.p + slot;
@@ -221,28 +227,47 @@ bool launch_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* 
   return cuda_ok(cudaGetLastError(), "kernel launch");
 }
 
+rf_status finish_host(const rf_model* m, rf_data* d, const Plan& plan, double* nll, double* grad, cudaStream_t st,
+                      bool in_place = false);
+
 // Host-buffer evaluation of the sets in `plan` (theta/out indexed by set).
-rf_status finish_host(const rf_model* m, rf_data* d, const Plan& plan, double* nll, double* grad, cudaStream_t st);
+// Each small copy beside the kernels costs 4 to 5 us of the call, whatever it
+// moves.  Up to kDirectBytes of results the kernels write them to the pinned
+// host buffers themselves (a set's block writes a few doubles, seen by the
+// host once the stream is done), and a single set's theta travels in the
+// kernels' arguments (not an extended model's, whose event kernel reads it
+// from memory).  us a call with copies / without, decay model, NLL of 1 toy
+// 48 / 38, 32 toys 52 / 47, 512 toys 179 / 173, 1024 toys 315 / 308 (56 KiB).
+constexpr size_t kDirectBytes = size_t(64) << 10;
 
 rf_status eval_host(const rf_model* m, rf_data* d, const Plan& plan, const double* theta, double* nll,
                     double* grad, cudaStream_t st) {
   if (!ensure_workspace(m, d)) return RF_E_OOM;
   Workspace& w = d->ws;
   const int P = m->m.prog.n_free, S = d->n_sets;
-  std::memcpy(w.h_theta.p, theta, sizeof(double) * S * P);
-  if (P > 0 && !cuda_ok(cudaMemcpyAsync(w.theta.p, w.h_theta.p, sizeof(double) * S * P, cudaMemcpyHostToDevice, st), "theta upload"))
+  const bool direct = sizeof(double) * S * (1 + P) <= kDirectBytes;
+  const bool by_value = S == 1 && !m->m.extended;
+  if (P > 0 && !by_value) {
+    std::memcpy(w.h_theta.p, theta, sizeof(double) * S * P);
+    if (!cuda_ok(cudaMemcpyAsync(w.theta.p, w.h_theta.p, sizeof(double) * S * P, cudaMemcpyHostToDevice, st), "theta upload"))
+      return RF_E_CUDA;
+  }
+  if (!launch_pass(m, d, plan, (const double*)w.theta.p, (double*)(direct ? w.h_out.p : w.out.p), (int32_t*)w.flags.p,
+                   grad != nullptr, st, -1, nullptr, direct ? (int32_t*)w.h_flags.p : nullptr,
+                   by_value ? theta : nullptr))
     return RF_E_CUDA;
-  if (!launch_pass(m, d, plan, (const double*)w.theta.p, (double*)w.out.p, (int32_t*)w.flags.p, grad != nullptr, st))
-    return RF_E_CUDA;
-  return finish_host(m, d, plan, nll, grad, st);
+  return finish_host(m, d, plan, nll, grad, st, direct);
 }
 
-// Downloads a pass's results (issued on st), waits, and fills nll / grad.
-rf_status finish_host(const rf_model* m, rf_data* d, const Plan& plan, double* nll, double* grad, cudaStream_t st) {
+// Downloads a pass's results (issued on st) unless they are written in place,
+// waits, and fills nll / grad.
+rf_status finish_host(const rf_model* m, rf_data* d, const Plan& plan, double* nll, double* grad, cudaStream_t st,
+                      bool in_place) {
   Workspace& w = d->ws;
   const int P = m->m.prog.n_free, S = d->n_sets;
-  if (!cuda_ok(cudaMemcpyAsync(w.h_out.p, w.out.p, sizeof(double) * S * (1 + P), cudaMemcpyDeviceToHost, st), "result download") ||
-      !cuda_ok(cudaMemcpyAsync(w.h_flags.p, w.flags.p, sizeof(int32_t) * S, cudaMemcpyDeviceToHost, st), "flag download") ||
+  if ((!in_place &&
+       (!cuda_ok(cudaMemcpyAsync(w.h_out.p, w.out.p, sizeof(double) * S * (1 + P), cudaMemcpyDeviceToHost, st), "result download") ||
+        !cuda_ok(cudaMemcpyAsync(w.h_flags.p, w.flags.p, sizeof(int32_t) * S, cudaMemcpyDeviceToHost, st), "flag download"))) ||
       !cuda_ok(cudaStreamSynchronize(st), "stream sync"))
     return RF_E_CUDA;
   const double* o = (const double*)w.h_out.p;

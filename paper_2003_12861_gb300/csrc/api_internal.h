@@ -166,8 +166,11 @@ constexpr int kPassSlots = 4;
 // dyn: null, or device counts {active sets, work items} that replace the
 // plan's (whose sets and items buffers then hold the device-compacted plan
 // of a device-resident fit); no active set skips the pass.
+// flags_out, theta1: null, or a host-buffer call's flags and its single set's
+// theta (Pass::flags_out, Pass::theta1).
 bool launch_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* d_theta, double* d_out,
-                 int32_t* d_flags, bool grad, cudaStream_t st, int slot = -1, const int32_t* dyn = nullptr);
+                 int32_t* d_flags, bool grad, cudaStream_t st, int slot = -1, const int32_t* dyn = nullptr,
+                 int32_t* flags_out = nullptr, const double* theta1 = nullptr);
 rf_status eval_host(const rf_model* m, rf_data* d, const Plan& plan, const double* theta, double* nll,
                     double* grad, cudaStream_t st);
 }  // namespace rf

@@ -286,6 +286,7 @@ __device__ void finish_param_point(const Program& P, const Pass& pass, int s, bo
     double* o = pass.out + (size_t)s * (1 + P.n_free);
     double ext = 0.0, dext = 0.0;
     if (P.ext && !bad) extended_term(P, pass, s, 0.0, &ext, &dext);
+    if (pass.flags_out) pass.flags_out[s] = pass.flags[s];
     o[0] = bad ? INFINITY : ext;
     if (pass.want_grad)
       for (int k = 0; k < P.n_free; ++k) o[1 + k] = k == P.ext_free ? dext : 0.0;
@@ -366,6 +367,7 @@ __global__ void __launch_bounds__(kK1Warps * 32) param_point_block_kernel(const 
   __shared__ EndFF endff[2];
   __shared__ ff geff[8];
   __shared__ int ffok;
+  __shared__ double th[kMaxFree];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if ((int)blockIdx.x >= (pass.dyn ? pass.dyn[0] : pass.n_active)) return;
   if (blockIdx.x == 0 && tid == 0) {
@@ -381,10 +383,10 @@ __global__ void __launch_bounds__(kK1Warps * 32) param_point_block_kernel(const 
     sbad = 0;
     ffok = 1;
   }
+  const int s = pass.sets[blockIdx.x];
+  if (tid < P.n_free) th[tid] = pass.n_theta1 ? pass.theta1[tid] : pass.theta[(size_t)s * P.n_free + tid];
   if (try_ff) ff_load_tables(T);
   __syncthreads();
-  const int s = pass.sets[blockIdx.x];
-  const double* th = pass.theta + (size_t)s * P.n_free;
   double* C = pass.consts + (size_t)s * P.n_const;
   if (try_ff) {
     // float-float path (k1_ff.cuh): the two range ends of the decay node on
@@ -891,6 +893,7 @@ __device__ void climb_tree(const Program& P, const Pass& pass, S& sm, int set, i
     if (tid == 0) {
       const int flag = pass.flags[set] + __ldcg(pass.tree_bad + root);
       pass.flags[set] = flag;
+      if (pass.flags_out) pass.flags_out[set] = flag;
       const double s0 = __ldcg(row) + __ldcg(row + Q);
       o[0] = flag ? INFINITY : ext - s0;
     } else if (pass.want_grad) {

@@ -53,6 +53,12 @@ struct Pass {
   // the device (sets and items then hold at least that many entries).  No
   // active set: the pass is skipped.
   const int32_t* dyn;
+  // Host-buffer calls on few sets.  flags_out: null, or where the sets' final
+  // flags go (out then is host memory too); n_theta1: 0, or a single set's
+  // theta passed by value in place of `theta`.
+  int32_t* flags_out;
+  int32_t n_theta1;
+  double theta1[kMaxFree];
 };
 
 // Resident blocks per SM the float-float kernels are compiled for (their
