@@ -9,6 +9,7 @@
 
 #include <cuda_runtime.h>
 
+#include "fp64_math.cuh"
 #include "rf_internal.h"
 
 namespace rf {
@@ -49,9 +50,9 @@ __device__ __forceinline__ double quotient(double t, const Divisor& d) {
 // that it depends on, and only their tangents are computed.  The others'
 // are zero; where arithmetic with that zero would give NaN (times an
 // infinity), the derivatives are marked not finite all the same.
-template <bool kDeriv>
+template <bool kDeriv, class M = LibMath>
 __device__ __forceinline__ int expr_eval(const Program& P, const PNode& q, const double* par, double x, double* f,
-                                         double* df) {
+                                         double* df, const M& mt = M()) {
   double v[kExprStack], d[kDeriv ? kExprStack : 1][kMaxPar];
   unsigned act[kDeriv ? kExprStack : 1];
   bool wild = false;  // a tangent left the finite range
@@ -84,7 +85,7 @@ __device__ __forceinline__ int expr_eval(const Program& P, const PNode& q, const
         for (unsigned m = ma; m; m &= m - 1) d[a][__ffs(m) - 1] = -d[a][__ffs(m) - 1];
         break;
       case RF_EX_EXP: {
-        const double r = exp(va);
+        const double r = mt.exp_(va);
         v[a] = r;
         if constexpr (kDeriv) wild |= not_finite(r);
         for (unsigned m = ma; m; m &= m - 1) d[a][__ffs(m) - 1] *= r;
@@ -137,7 +138,7 @@ __device__ __forceinline__ int expr_eval(const Program& P, const PNode& q, const
       }
       default: {  // RF_EX_POW: a^b = exp(b log a), a > 0
         if (!(va > 0.0)) return 1;
-        const double la = log(va), r = exp(vb * la);
+        const double la = log(va), r = mt.exp_(vb * la);
         v[a] = r;
         if constexpr (kDeriv) wild |= not_finite(r) || not_finite(la) || not_finite(vb);
         for (unsigned m = ma | mb; m; m &= m - 1) {

@@ -569,9 +569,9 @@ static_assert(kSlowZ == -7.0, "is_slow_z holds its bits");
 // in per-thread memory, and no node divides by what it multiplied with
 // (kKept; the float-float kernels' rare events compute it again, as those
 // arrays would cost their event loop 1 % of its time).
-template <bool kFull, bool kGrad, bool kExpr = false, bool kKept = true>
+template <bool kFull, bool kGrad, bool kExpr = false, bool kKept = true, class M = LibMath>
 __device__ bool eval_generic(const Program& P, const double* __restrict__ C, const double* x, double* acc,
-                             LogProd64& L, int* bad, int n0 = 0, int n1 = -1) {
+                             LogProd64& L, int* bad, int n0 = 0, int n1 = -1, const M& mt = M()) {
   double v[kMaxPdf];
   constexpr bool kKeep = kGrad && kKept;
   double w1[kKeep ? kMaxPdf : 1];             // per node: u, or the unnormalised value
@@ -586,10 +586,10 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
       case GAUSS: {
         const double u = (x[q.col] - c[0]) * c[1];
         if constexpr (kKeep) w1[n] = u;
-        v[n] = exp(-0.5 * u * u) * c[2];
+        v[n] = mt.exp_(-0.5 * u * u) * c[2];
         break;
       }
-      case EXPO: v[n] = exp(c[0] * (x[q.col] - c[1])) * c[2]; break;
+      case EXPO: v[n] = mt.exp_(c[0] * (x[q.col] - c[1])) * c[2]; break;
       case GAUSSEXP: {
         const double u = (x[q.col] - c[0]) * c[1], s = c[2];
         const double z = (s - u) * kSqrt1_2;
@@ -597,11 +597,12 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
         double f;
         if constexpr (!kFull) {
           if (is_slow_z(z)) return false;
-          f = exp(s * (0.5 * s - u));
+          f = mt.exp_(s * (0.5 * s - u));
         } else {
-          const bool right = z > 0.0;
-          const double g = kGrad || right ? exp(-0.5 * u * u) : 0.0;
-          f = right ? 0.5 * g * erfcx(z) : 0.5 * exp(s * (0.5 * s - u)) * erfc(z);
+          const bool right = __double2hiint(z) >= 0;
+          const double g = kGrad || right ? mt.exp_(-0.5 * u * u) : 0.0;
+          const double w = right ? g : mt.exp_(s * (0.5 * s - u));
+          f = 0.5 * w * mt.tail(z, right);
           if constexpr (kKeep) {
             w2[n] = g;
             f1[n] = f;
@@ -637,13 +638,13 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
       }
       case POISSON: {
         const double k = fmin(floor(x[q.col]), q.hi - 1.0);
-        v[n] = exp(k * c[1] - c[0] - lgamma(k + 1.0)) * c[3];
+        v[n] = mt.exp_(k * c[1] - c[0] - lgamma(k + 1.0)) * c[3];
         break;
       }
       case EXPR: {
         if constexpr (kExpr) {
           double f;
-          v[n] = expr_eval<kGrad>(P, q, c + 1 + q.n_par, x[q.col], &f, dex + (kGrad ? q.slot0 : 0)) != 1 ? f * c[0] : NAN;
+          v[n] = expr_eval<kGrad>(P, q, c + 1 + q.n_par, x[q.col], &f, dex + (kGrad ? q.slot0 : 0), mt) != 1 ? f * c[0] : NAN;
           if constexpr (kGrad) w1[n] = f;
         }
         break;
@@ -786,7 +787,7 @@ struct SmemT {
   int item;
   int last;
 };
-using Smem = SmemT<int, kPerLane * 32>;
+using Smem = SmemT<uint16_t, kPerLane * 32>;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -1006,18 +1007,21 @@ __device__ void finish_unit(const Program& P, const Pass& pass, Smem& sm, const 
 // converged; the lane order of additions is still fixed by the data alone.
 // The next unit is claimed after the unit's events, when the other blocks
 // have had their share.
-// Bound by the FP64 unit (84 % busy, 91 FP64 instructions an event for the
-// decay model).  Before / after the split into parts, one evaluation of a
-// program per event and the values kept for the gradient pass: decay model
-// 1e4 events 203 -> 41 us, 1e6 285 -> 217, 4e6 862 -> 705; program model 1e4
-// 629 -> 54, 1e6 822 -> 355.
+// Bound by the FP64 unit.  First with the split into parts, one evaluation of
+// a program per event and the values kept for the gradient pass, then with
+// the functions of fp64_math.cuh: decay model 1e4 events 203 -> 41 -> 39 us,
+// 1e6 285 -> 217 -> 187, 4e6 862 -> 705 -> 601; program model 1e4 629 -> 54
+// -> 51, 1e6 822 -> 355 -> 329.
 template <bool kGrad, bool kExpr>
 __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__ Program P,
                                                          const __grid_constant__ Columns cols, Pass pass) {
   __shared__ Smem sm;
+  __shared__ double2 exp_tab[256];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_units = (pass.dyn ? pass.dyn[1] : pass.n_items) * pass.parts;
   if (n_units == 0) return;
+  for (int i = tid; i < 256; i += kLanes) exp_tab[i] = ((const double2*)kExp64)[i];
+  const TableMath mt{exp_tab};
   pdl_wait();
   const int per_lane = kPerLane / pass.parts;
   if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
@@ -1041,11 +1045,11 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
       bool slow = false;
       if (e < s_end) {
         for (int c = 0; c < P.n_obs; ++c) x[c] = load_col(cols, c, e);
-        slow = !eval_generic<false, kGrad, kExpr>(P, sm.C, x, acc, L, &bad);
+        slow = !eval_generic<false, kGrad, kExpr>(P, sm.C, x, acc, L, &bad, 0, -1, mt);
       }
       if (P.has_slow) {
         const unsigned b = __ballot_sync(0xffffffffu, slow);
-        if (slow) sm.queue[warp][qcnt + __popc(b & ((1u << lane) - 1u))] = (int)(e - base);
+        if (slow) sm.queue[warp][qcnt + __popc(b & ((1u << lane) - 1u))] = (uint16_t)(e - base);
         qcnt += __popc(b);
       }
     }
@@ -1054,7 +1058,7 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
     for (int j = lane; j < qcnt; j += 32) {
       const int64_t e = base + sm.queue[warp][j];
       for (int c = 0; c < P.n_obs; ++c) x[c] = load_col(cols, c, e);
-      eval_generic<true, kGrad, kExpr>(P, sm.C, x, acc, L, &bad);
+      eval_generic<true, kGrad, kExpr>(P, sm.C, x, acc, L, &bad, 0, -1, mt);
     }
     if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
     acc[0] += logprod64_log(L);

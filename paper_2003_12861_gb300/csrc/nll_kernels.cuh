@@ -81,14 +81,15 @@ __host__ __device__ constexpr int ff_min_blocks(int shape) { return shape == SHA
 //
 // The generic kernel's events are bound by the FP64 unit (1 us a warp), and
 // per unit it pays a pass over the queued events, a logarithm and the sums.
-// It splits chunks, up to 16 ways, until there are six units for each SM:
-// us with 1 | 2 | 4 | 8 | 16 parts for the decay model with the 8-block grid,
-// 1e4 events 181 | 100 | 69 | 47 | 41, 3e5 193 | 115 | 89 | 91 | 125, 1e6
-// 244 | 226 | 217 | 243 | 351, 4e6 705 | 681 | 760 | 908 | 1269; for the
-// program model 1e4 483 | 252 | 137 | 81 | 54, 1e6 597 | 416 | 355 | 347 |
-// 396, 4e6 1300 | 1250 | 1314 | 1289 | 1381.
+// It splits chunks, up to 16 ways, until there are three and a half units
+// for each SM: us with 1 | 2 | 4 | 8 | 16 parts for the decay model, 1e4
+// events 172 | 96 | 65 | 45 | 39, 3e5 182 | 109 | 82 | 79 | 104, 6e5 183 |
+// 131 | 117 | 137 | 199, 1e6 224 | 195 | 187 | 203 | 284, 2e6 348 | 326 |
+// 345 | 394 | 527, 4e6 601 | 582 | 633 | 750 | 1015; for the program model
+// 1e4 418 | 220 | 121 | 74 | 51, 6e5 434 | 270 | 203 | 210 | 239, 2e6 700 |
+// 622 | 630 | 655 | 674, 4e6 1206 | 1206 | 1227 | 1214 | 1311.
 constexpr int kMaxParts = 4, kMaxPartsGeneric = 16;
-constexpr int kRefSMs = 152, kGenericUnits = kRefSMs * 6;
+constexpr int kRefSMs = 152, kGenericUnits = kRefSMs * 7 / 2;
 inline int parts_for(int64_t total_chunks, int shape) {
   if (shape == SHAPE_GENERIC) {
     int P = 1;
