@@ -374,11 +374,14 @@ __global__ void __launch_bounds__(kK1Warps * 32) param_point_block_kernel(const 
     for (int i = 0; i < (pass.n_counters > 1 ? pass.n_counters : 1); ++i) pass.counter[i] = 0;
     if (pass.slow) *pass.slow = 0ull;
   }
-  // The event kernel may launch once this kernel has started (FP64 path) or
-  // once the float-float chain is done: its waiting blocks would otherwise
-  // share the issue slots that the chain's single warp depends on.
+  // The event kernel may launch once the constants are there but for their
+  // copy out (FP64 path) or once the float-float chain is done.  Earlier, its
+  // waiting blocks share the issue slots that the chain's single warp depends
+  // on, and they are placed around this kernel's blocks: with two of those on
+  // some SMs and one or none on others the units end up on half of the GPU
+  // (decay model on the interpreter, 192 toys: 449 us a pass; with the launch
+  // here at the end 274, 64 toys 165 -> 128, one 51 -> 50).
   const bool try_ff = decay_ff_eligible(P, pass);
-  if (!try_ff) pdl_launch_dependents();
   if (tid == 0) {
     sbad = 0;
     ffok = 1;
@@ -493,6 +496,7 @@ __global__ void __launch_bounds__(kK1Warps * 32) param_point_block_kernel(const 
     __syncthreads();
     ff_convert_K(shape, Ks, out, tid, blockDim.x);
   }
+  if (!try_ff) pdl_launch_dependents();
   for (int i = tid; i < P.n_const; i += blockDim.x) C[i] = Cs[i];
   if (tid == 0) finish_param_point(P, pass, s, sbad != 0, Cs, true);
 }
@@ -1344,6 +1348,18 @@ __global__ void __launch_bounds__(kLanes, ff_min_blocks(kShape)) events_ff(const
 
 }  // namespace
 
+// Up to this many active sets K1 runs one block per set (latency), beyond
+// one thread per set (throughput).  us a pass of toys of 6000 events, thread
+// form / block form: decay 256 toys 79 / 67, 768 114 / 109, 1024 138 / 139;
+// product model 256 183 / 118, 768 289 / 250; the interpreter 256 342 / 331,
+// 768 875 / 813; Gauss + line, whose constants are the cheapest, 384 65 / 59,
+// 512 74 / 78.  Beside another pass (the halves of a pipelined fit) the
+// blocks compete with its event pass: 256, as measured there.
+static int block_k1_sets(const Pass& pass) {
+  if (pass.beside) return 256;
+  return pass.ff_shape == SHAPE_SUM_GAUSS_POLY1 ? 384 : 768;
+}
+
 void launch_param_point(const Program& P, const Pass& pass, cudaStream_t st) {
   note_launches(1, st);
   if (pass.n_active > 0 && P.has_expr) {
@@ -1352,7 +1368,7 @@ void launch_param_point(const Program& P, const Pass& pass, cudaStream_t st) {
   }
   // In the rounds of a device-resident fit (dyn counts) nothing runs beside
   // K1, and a block per set finishes sooner for any number of sets.
-  if (pass.n_active > 0 && (pass.n_active <= kBlockK1MaxSets || pass.dyn)) {
+  if (pass.n_active > 0 && (pass.n_active <= block_k1_sets(pass) || pass.dyn)) {
     param_point_block_kernel<false><<<pass.n_active, kK1Warps * 32, 0, st>>>(P, pass);
     return;
   }

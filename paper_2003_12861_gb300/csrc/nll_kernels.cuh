@@ -53,6 +53,7 @@ struct Pass {
   // the device (sets and items then hold at least that many entries).  No
   // active set: the pass is skipped.
   const int32_t* dyn;
+  int32_t beside;           // 1: runs beside another pass on another stream (a pipelined fit's halves)
   // Host-buffer calls on few sets.  flags_out: null, or where the sets' final
   // flags go (out then is host memory too); n_theta1: 0, or a single set's
   // theta passed by value in place of `theta`.
