@@ -12,6 +12,7 @@
 #include "api_internal.h"
 #include "nll_ff.cuh"
 #include "nll_kernels.cuh"
+#include "workspace.h"
 
 namespace rf {
 
@@ -124,46 +125,31 @@ void note_launches(int n, cudaStream_t st) {
 
 bool ensure_workspace(const rf_model* m, rf_data* d) {
   Workspace& w = d->ws;
-  const Program& P = m->m.prog;
-  const int Q = 1 + P.n_slots;
-  const int gen_parts = parts_for(d->total_chunks, SHAPE_GENERIC);
-  if (w.ready && w.n_const == P.n_const && w.n_free == P.n_free && w.Q == Q &&
-      (m->m.shape == SHAPE_GENERIC ? gen_parts == 1 || w.gen_part.p : w.ffc.p != nullptr))
-    return true;
-  const size_t S = d->n_sets;
-  const size_t nodes = (size_t)std::max<int64_t>(1, d->total_nodes);
-  bool ok = w.consts.ensure(sizeof(double) * S * std::max(1, P.n_const)) &&
-            w.theta.ensure(sizeof(double) * S * std::max(1, P.n_free)) &&
-            w.out.ensure(sizeof(double) * S * (1 + P.n_free)) && w.flags.ensure(sizeof(int32_t) * S) &&
-            w.tree.ensure(sizeof(double) * std::max<int64_t>(1, d->total_nodes) * 2 * Q) &&
-            w.tree_bad.ensure(sizeof(int32_t) * std::max<int64_t>(1, d->total_nodes)) &&
-            w.tickets.ensure(sizeof(int32_t) * std::max<int64_t>(1, d->total_nodes)) &&
-            w.counter.ensure(sizeof(int32_t)) && w.slow.ensure(sizeof(unsigned long long)) &&
-            w.slot_counter.ensure(sizeof(int32_t) * kPassSlots) &&
-            w.slot_slow.ensure(sizeof(unsigned long long) * kPassSlots) &&
-            (m->m.shape != SHAPE_GENERIC || gen_parts == 1 ||
-             (w.gen_part.ensure(sizeof(double) * nodes * gen_parts * 2 * Q) &&
-              w.gen_info.ensure(sizeof(int32_t) * nodes * gen_parts))) &&
-            (m->m.shape == SHAPE_GENERIC ||
-             (w.ffc.ensure(sizeof(float) * S * kFFConst) &&
-              w.part_m.ensure(sizeof(float) * nodes * kMaxParts * kPartFloats) &&
-              w.part_fb.ensure(sizeof(double) * nodes * kMaxParts * Q) &&
-              w.part_info.ensure(sizeof(int32_t) * nodes * kMaxParts))) &&
-            w.h_theta.ensure(sizeof(double) * S * std::max(1, P.n_free)) &&
-            w.h_out.ensure(sizeof(double) * S * (1 + P.n_free)) && w.h_flags.ensure(sizeof(int32_t) * S);
+  const WorkspaceBytes b =
+      workspace_bytes(m->m.prog, m->m.shape, d->n_sets, d->total_nodes, d->total_chunks, kFFConst);
+  const bool ok = w.consts.ensure(b.consts) && w.theta.ensure(b.theta) && w.out.ensure(b.out) &&
+                  w.flags.ensure(b.flags) && w.tree.ensure(b.tree) && w.tree_bad.ensure(b.node_words) &&
+                  w.counter.ensure(sizeof(int32_t)) && w.slow.ensure(sizeof(unsigned long long)) &&
+                  w.slot_counter.ensure(sizeof(int32_t) * kPassSlots) &&
+                  w.slot_slow.ensure(sizeof(unsigned long long) * kPassSlots) &&
+                  (b.ffc == 0 || w.ffc.ensure(b.ffc)) && (b.part_m == 0 || w.part_m.ensure(b.part_m)) &&
+                  (b.part_fb == 0 || w.part_fb.ensure(b.part_fb)) &&
+                  (b.part_info == 0 || w.part_info.ensure(b.part_info)) && w.h_theta.ensure(b.theta) &&
+                  w.h_out.ensure(b.out) && w.h_flags.ensure(b.flags);
   if (!ok) return false;
-  if (!cuda_ok(cudaMemset(w.tickets.p, 0, sizeof(int32_t) * std::max<int64_t>(1, d->total_nodes)), "ticket reset"))
-    return false;
+  if (!w.tickets.p) {  // a dataset's nodes are fixed; the kernels leave the tickets at zero
+    if (!w.tickets.ensure(b.node_words)) return false;
+    if (!cuda_ok(cudaMemset(w.tickets.p, 0, b.node_words), "ticket reset")) {
+      w.tickets.release();
+      return false;
+    }
+  }
   if (!d->all_plan_ready) {
     std::vector<int32_t> all(d->n_sets);
     for (int s = 0; s < d->n_sets; ++s) all[s] = s;
     if (!build_plan(d, all, &d->all_plan)) return false;
     d->all_plan_ready = true;
   }
-  w.n_const = P.n_const;
-  w.n_free = P.n_free;
-  w.Q = Q;
-  w.ready = true;
   return true;
 }
 
@@ -191,8 +177,8 @@ Pass make_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* d_
   p.ff_shape = m->m.shape;
   p.ffc = m->m.shape == SHAPE_GENERIC ? nullptr : (float*)w.ffc.p;
   p.part_m = (float*)w.part_m.p;
-  p.part_fb = (double*)(m->m.shape == SHAPE_GENERIC ? w.gen_part.p : w.part_fb.p);
-  p.part_info = (int32_t*)(m->m.shape == SHAPE_GENERIC ? w.gen_info.p : w.part_info.p);
+  p.part_fb = (double*)w.part_fb.p;
+  p.part_info = (int32_t*)w.part_info.p;
   p.parts = parts_for(d->total_chunks, m->m.shape);
   p.pairs = nullptr;
   return p;

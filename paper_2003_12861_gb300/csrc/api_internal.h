@@ -40,18 +40,16 @@ struct Plan {
   int32_t n_active = 0, n_items = 0;
 };
 
-// Per-dataset evaluation buffers for the model last used with it.
 // Segments of the streamed host-column pass (rf_nll_grad_stream).
 constexpr int kMaxSegments = 16;
 // Compute streams the segments rotate over, so that one segment's pass
 // starts while the previous one finishes its last work units.
 constexpr int kCompStreams = 4;
 
+// A dataset's evaluation buffers, grown to the largest that a model evaluated
+// on it needs (ensure_workspace; sizes in workspace.h).
 struct Workspace {
-  bool ready = false;
-  int n_const = -1, n_free = -1, Q = -1;
   DevBuf consts, theta, out, flags, tree, tree_bad, tickets, counter, slow, ffc, part_m, part_fb, part_info;
-  DevBuf gen_part, gen_info;  // part records of the generic kernel
   // work and slow-event counters of passes that may run concurrently on
   // other streams (launch_pass with slot >= 0)
   DevBuf slot_counter, slot_slow;
