@@ -670,11 +670,13 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   int dev_id = 0, max_optin = 0;
   cudaGetDevice(&dev_id);
   cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev_id);
+  // The attribute is the kernel's, for every model in the process: once the
+  // device's maximum, not this model's size (a smaller model created later
+  // took a larger one's launches away).
   if (m->smem > (size_t)max_optin ||
-      !cuda_ok(cudaFuncSetAttribute(binned_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem),
+      !cuda_ok(cudaFuncSetAttribute(binned_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin),
                "binned smem") ||
-      !cuda_ok(cudaFuncSetAttribute(binned_expected_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)m->smem),
+      !cuda_ok(cudaFuncSetAttribute(binned_expected_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin),
                "binned smem")) {
     delete m;
     set_error("rf_binned_create: the model needs more shared memory than a block has");
