@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <list>
 #include <vector>
 
 #include "api_internal.h"
@@ -101,7 +102,8 @@ struct BinnedDev {
   const GradRec* grad;
 };
 
-// The intermediate results of a pass for up to `cap` datasets, dataset-major.
+// The intermediate results of a pass for up to rf_binned::cap datasets,
+// dataset-major.
 struct BinnedScratch {
   float4* pt;      // per parameter: theta and g as float pairs
   double* dgk;     // g'
@@ -414,7 +416,7 @@ __global__ void __launch_bounds__(kBinnedThreads) binned_expected_kernel(const B
   double* th = smem;
   double* F = th + m.n_params;
   double* gk = F + m.n_samples;
-  double* nu_e = scratch + (size_t)blockIdx.x * (m.n_entries + m.n_hs);
+  double* nu_e = scratch + (size_t)blockIdx.x * m.n_entries;
   for (int set = blockIdx.x; set < n_sets; set += gridDim.x) {
     sample_factors(m, theta + (size_t)set * m.n_params, th, gk, F);
     entry_rates(m, th, gk, F, nu_e);
@@ -434,16 +436,36 @@ __global__ void __launch_bounds__(kBinnedThreads) binned_expected_kernel(const B
 
 // ---------------------------------------------------------------- handle
 
+// A buffer that grows and keeps what it had (at most as much again, if it
+// grows at least twofold), as queued work and captured graphs use it.  The
+// stream may be capturing: the allocation is no part of that.
+struct GrowBuf {
+  std::list<rf::DevBuf> kept;  // the last one is in use
+  void* p() const { return kept.empty() ? nullptr : kept.back().p; }
+  size_t bytes() const { return kept.empty() ? 0 : kept.back().bytes; }
+  bool grow(size_t b) {
+    if (b <= bytes()) return true;
+    kept.emplace_back();
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const bool ok = kept.back().ensure(b);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!ok) kept.pop_back();
+    return ok;
+  }
+};
+
 struct rf_binned {
   int32_t n_bins = 0, n_samples = 0, n_params = 0, n_mods = 0, n_entries = 0, n_hs = 0;
   rf::DevBuf bin0, nb, eofs, esample, nominal, smod_start, shs_start, shs, hs_param, hs_ofs, coef, tbase, g_sample,
       bin_start, bin_entry, pmod_start, constrained, nominal_f, coef_f, coef_af, coef_bf, shs_k, shs_ofs, factor, grad;
-  rf::DevBuf scratch, work, counts, theta, out, flags, sets, io;
+  rf::DevBuf counts, theta, out, flags, sets, io;
+  GrowBuf work, scratch;  // intermediate results of the passes, of the expected counts
   rf::HostBuf h_out, h_flags, h_theta, h_sets, h_io;
   rf::BinnedDev dev{};
   rf::BinnedScratch ws{};
-  int grid = 0;  // blocks of the expected-counts kernel
-  int cap = 0;   // datasets a pass takes at once
+  int grid = 0;  // most blocks of the expected-counts kernel
+  int cap = 0;   // datasets a pass takes at once: those that `work` has room for
   size_t smem = 0;
 };
 
@@ -475,10 +497,50 @@ void launch_chained(void (*kernel)(Params...), dim3 grid, int threads, size_t sm
   cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Bytes of a dataset's intermediate results.
+size_t work_per_set(const rf_binned* m) {
+  return 24 * (size_t)std::max(1, m->n_params) + 24 * (size_t)m->n_samples + 8 * (size_t)m->n_entries +
+         16 * (size_t)m->n_bins + 8 * (size_t)std::max(1, m->n_hs);
+}
+
+// Room for the intermediate results of n datasets, of 1024 or 256 MB at most,
+// one at least (n <= 0: of the datasets that 8 MB hold).  A model starts with
+// 8 MB (50 datasets of the 28-channel model, whose 160 MB for 1024 would lie
+// idle beside models that only see a few) and grows to what a call has, at
+// least twofold.  Without memory a call goes on in groups of `cap`.
+bool reserve_sets(rf_binned* m, int n) {
+  const size_t per_set = work_per_set(m);
+  const auto held = [&](size_t bytes) { return (int)std::max<size_t>(1, std::min<size_t>(1024, bytes / per_set)); };
+  const int most = held((size_t)256 << 20);
+  if (m->cap > 0 && std::min(n, most) <= m->cap) return true;
+  const int cap = std::min(most, n > 0 ? std::max(n, 2 * m->cap) : held((size_t)8 << 20));
+  if (!m->work.grow(per_set * (size_t)cap)) return false;
+  m->cap = cap;
+  char* p = (char*)m->work.p();  // (16-byte items first)
+  auto take = [&](size_t bytes) {
+    char* q = p;
+    p += bytes * (size_t)cap;
+    return (void*)q;
+  };
+  const size_t P = (size_t)std::max(1, m->n_params), S = (size_t)m->n_samples, E = (size_t)m->n_entries,
+               B = (size_t)m->n_bins, H = (size_t)std::max(1, m->n_hs);
+  m->ws.pt = (float4*)take(16 * P);
+  m->ws.dgk = (double*)take(8 * P);
+  m->ws.F = (double*)take(8 * S);
+  m->ws.Ssum = (double*)take(8 * S);
+  m->ws.Ff = (float2*)take(8 * S);
+  m->ws.nu_e = (float2*)take(8 * E);
+  m->ws.W = (float2*)take(8 * B);
+  m->ws.term = (double*)take(8 * B);
+  m->ws.T = (double*)take(8 * H);
+  return true;
+}
+
 rf_status launch_binned(rf_binned* m, int32_t n_sets, const double* d_counts, const double* d_theta, double* d_out,
                         int32_t* d_flags, cudaStream_t st, const int32_t* d_sets = nullptr) {
   const BinnedDev& D = m->dev;
   const int P = D.n_params;
+  reserve_sets(m, n_sets);
   for (int s0 = 0; s0 < n_sets; s0 += m->cap) {
     const int n = std::min(n_sets - s0, m->cap);
     const double* th = d_theta + (size_t)s0 * P;
@@ -685,34 +747,9 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, binned_expected_kernel, kBinnedThreads, m->smem);
   m->grid = sm_count() * std::max(1, per_sm);
-  // A pass's intermediate results: datasets in groups that need at most
-  // 256 MB (1024 at most, one at least).
-  const size_t P_ = (size_t)std::max(1, n_params), S_ = (size_t)n_samples, E_ = (size_t)total, B_ = (size_t)n_bins,
-               H_ = (size_t)std::max(1, n_hs);
-  const size_t per_set = 24 * P_ + 24 * S_ + 8 * E_ + 16 * B_ + 8 * H_;
-  m->cap = (int)std::max<size_t>(1, std::min<size_t>(1024, ((size_t)256 << 20) / per_set));
-  // (the expected counts' entry rates: per block n_entries + n_hs doubles)
-  if (!ok || !m->scratch.ensure(sizeof(double) * (size_t)m->grid * (E_ + H_)) ||
-      !m->work.ensure(per_set * (size_t)m->cap)) {
+  if (!ok || !m->scratch.grow(sizeof(double) * (size_t)total) || !reserve_sets(m, 0)) {
     delete m;
     return RF_E_OOM;
-  }
-  {
-    char* p = (char*)m->work.p;  // (16-byte items first)
-    auto take = [&](size_t bytes) {
-      char* q = p;
-      p += bytes * (size_t)m->cap;
-      return (void*)q;
-    };
-    m->ws.pt = (float4*)take(16 * P_);
-    m->ws.dgk = (double*)take(8 * P_);
-    m->ws.F = (double*)take(8 * S_);
-    m->ws.Ssum = (double*)take(8 * S_);
-    m->ws.Ff = (float2*)take(8 * S_);
-    m->ws.nu_e = (float2*)take(8 * E_);
-    m->ws.W = (float2*)take(8 * B_);
-    m->ws.term = (double*)take(8 * B_);
-    m->ws.T = (double*)take(8 * H_);
   }
   BinnedDev& D = m->dev;
   D.n_bins = n_bins;
@@ -832,9 +869,16 @@ rf_status rf_binned_expected(rf_binned* m, int32_t n_sets, const double* d_theta
     return RF_E_INVALID;
   }
   if (n_sets == 0) return RF_OK;
+  // A block's entry rates are n_entries doubles; without memory for all blocks,
+  // as many as there is room for.
+  const size_t per_block = sizeof(double) * (size_t)m->n_entries;
+  int grid = std::min(n_sets, m->grid);
+  if (m->scratch.bytes() < per_block * (size_t)grid)
+    m->scratch.grow(per_block * std::min((size_t)m->grid, std::max((size_t)grid, 2 * m->scratch.bytes() / per_block)));
+  grid = (int)std::min((size_t)grid, m->scratch.bytes() / per_block);
   note_launches(1, (cudaStream_t)stream);
-  binned_expected_kernel<<<std::min(n_sets, m->grid), kBinnedThreads, m->smem, (cudaStream_t)stream>>>(
-      m->dev, n_sets, d_theta, d_nu, (double*)m->scratch.p);
+  binned_expected_kernel<<<grid, kBinnedThreads, m->smem, (cudaStream_t)stream>>>(m->dev, n_sets, d_theta, d_nu,
+                                                                                  (double*)m->scratch.p());
   return cuda_ok(cudaGetLastError(), "binned launch") ? RF_OK : RF_E_CUDA;
 }
 
