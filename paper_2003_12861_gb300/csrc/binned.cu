@@ -395,11 +395,10 @@ __global__ void __launch_bounds__(kGradThreads) binned_grad_kernel(const BinnedD
 #pragma unroll 4
     for (int j = m.pmod_start[k] + l; j < j1; j += kGradLanes) {
       const GradRec r = m.grad[j];
-      const double x = r.kind == MOD_HISTOSYS ? F[r.sample] : S[r.sample];
-      double y;
+      double x = r.kind == MOD_HISTOSYS ? F[r.sample] : S[r.sample], y = 1.0;
       if (r.kind == MOD_HISTOSYS) y = T[r.hs];
       else if (r.kind == MOD_NORMSYS) y = fma(r.b, dg, r.a);
-      else y = 1.0 / a;
+      else x /= a;  // (one rounding; by the reciprocal it would be two)
       g = fma(x, y, g);
     }
   }
