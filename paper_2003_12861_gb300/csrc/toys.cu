@@ -872,10 +872,11 @@ rf_status rf_hist64(const rf_model* m, const rf_data* d, int32_t col, float* d_o
   const cudaStream_t st = (cudaStream_t)stream;
   const double lo = m->m.obs_lo[col], hi = m->m.obs_hi[col], scale = 64.0 / (hi - lo);
   // x, lo and scale as floats, the difference and the product: at most 2^-23
-  // of |x| + |lo|, in bins, and 2^-22 of the coordinate (below 128); four times
-  // that (beyond 0.5, every event takes the FP64 expression).
+  // of |x| + |lo| and, for an x that is no normal float, 2^-126 (hist_float
+  // takes it as zero), in bins, and 2^-22 of the coordinate (below 128); four
+  // times that (beyond 0.5, every event takes the FP64 expression).
   const double far = std::max(std::fabs(lo), std::fabs(hi)) + (hi - lo);
-  const float reach = (float)std::min(1.0, 4.0 * (2.0 * far * scale * 0x1p-23 + 128.0 * 0x1p-22));
+  const float reach = (float)std::min(1.0, 4.0 * ((2.0 * far * 0x1p-23 + 0x1p-126) * scale + 128.0 * 0x1p-22));
   // Blocks per set: 8 resident blocks an SM fill the GPU; a block takes at
   // least 16384 events (64 a thread), below which a second one gains nothing.
   const int64_t per_set = (d->n_events + d->n_sets - 1) / d->n_sets;
