@@ -587,6 +587,7 @@ int bias_chunk(int batch) { return std::max(128, (batch + 15) / 16); }
 
 bool mlp_reserve(rf_mlp* n, int batch) {
   if (batch <= n->cap) return true;
+  n->cap = 0;  // (a buffer that cannot grow is lost with what it had)
   int64_t act = 0, z = 0, part = 0;
   const int wmax = *std::max_element(n->dims.begin(), n->dims.end());
   const int nout = n->dims.back();
