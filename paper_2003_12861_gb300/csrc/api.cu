@@ -204,7 +204,7 @@ bool launch_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* 
     std::memcpy(pass.theta1, theta1, sizeof(double) * m->m.prog.n_free);
   }
   if (slot >= 0 && slot < kPassSlots) {
-    pass.beside = 1;
+    pass.beside = slot_beside(slot) ? 1 : 0;
     pass.counter = (int32_t*)d->ws.slot_counter.p + slot;
     pass.slow = (unsigned long long*)d->ws.slot_slow.p + slot;
   }

@@ -161,6 +161,10 @@ bool ensure_workspace(const rf_model* m, rf_data* d);
 // kPassSlots) gives the pass its own work and slow-event counters, for
 // passes over disjoint sets that run at the same time on different streams.
 constexpr int kPassSlots = 4;
+// Whether a slot's pass has another one beside it (Pass::beside): a fit's two
+// halves do (slots 0 and 1), its whole-batch passes (2) and device rounds (3)
+// run alone, as the passes without a slot.
+constexpr bool slot_beside(int slot) { return slot == 0 || slot == 1; }
 // dyn: null, or device counts {active sets, work items} that replace the
 // plan's (whose sets and items buffers then hold the device-compacted plan
 // of a device-resident fit); no active set skips the pass.
