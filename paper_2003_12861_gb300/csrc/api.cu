@@ -137,6 +137,7 @@ bool ensure_workspace(const rf_model* m, rf_data* d) {
                   (b.part_info == 0 || w.part_info.ensure(b.part_info)) && w.h_theta.ensure(b.theta) &&
                   w.h_out.ensure(b.out) && w.h_flags.ensure(b.flags);
   if (!ok) return false;
+  const bool first = !w.tickets.p || !d->all_plan_ready;
   if (!w.tickets.p) {  // a dataset's nodes are fixed; the kernels leave the tickets at zero
     if (!w.tickets.ensure(b.node_words)) return false;
     if (!cuda_ok(cudaMemset(w.tickets.p, 0, b.node_words), "ticket reset")) {
@@ -150,7 +151,9 @@ bool ensure_workspace(const rf_model* m, rf_data* d) {
     if (!build_plan(d, all, &d->all_plan)) return false;
     d->all_plan_ready = true;
   }
-  return true;
+  // The tickets and the plan are written on the legacy stream, which a pass on
+  // a non-blocking stream would not wait for: done before the first one starts.
+  return !first || cuda_ok(cudaStreamSynchronize(nullptr), "workspace");
 }
 
 Pass make_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* d_theta, double* d_out,
