@@ -95,7 +95,8 @@ struct BinnedDev {
   const float2* coef_bf;
   const int32_t* bin_start;   // per bin: its entries (CSR, sample order)
   const int32_t* bin_entry;
-  const int32_t* pmod_start;  // per parameter: its modifiers (CSR, modifier order; `grad`)
+  const int32_t* pmod_start;  // per parameter: its modifiers (CSR, normfactors first, modifier order; `grad`)
+  const int32_t* pmod_norm;   // per parameter: the end of its normfactors
   const int32_t* constrained;
   // The modifiers as records in the order they are summed.
   const FactorRec* factor;
@@ -360,6 +361,9 @@ __global__ void __launch_bounds__(kBinnedThreads2) binned_sums_kernel(const Binn
 // others 16 parameters each, eight lanes a parameter: its modifiers lane by
 // lane, the lanes by butterfly, then its constraint.
 constexpr int kGradThreads = 128, kGradLanes = 8, kGradPer = kGradThreads / kGradLanes;
+// Out of line: inlined, every warp would divide (an FP64 division on each of
+// them takes as long as the kernel) and select.
+__device__ __noinline__ double divided(double x, double a) { return x / a; }
 __global__ void __launch_bounds__(kGradThreads) binned_grad_kernel(const BinnedDev m, const BinnedScratch w,
                                                                    const double* theta, double* out,
                                                                    const int32_t* flags) {
@@ -391,15 +395,15 @@ __global__ void __launch_bounds__(kGradThreads) binned_grad_kernel(const BinnedD
     const double* T = w.T + (size_t)set * m.n_hs;
     a = th[k];
     const double dg = w.dgk[(size_t)set * m.n_params + k];
-    const int j1 = m.pmod_start[k + 1];
+    const int j0 = m.pmod_norm[k], j1 = m.pmod_start[k + 1];
+    // the normfactors' sums, divided by a once
+    for (int j = m.pmod_start[k] + l; j < j0; j += kGradLanes) g += S[m.grad[j].sample];
+    if (m.pmod_start[k] + l < j0) g = divided(g, a);
 #pragma unroll 4
-    for (int j = m.pmod_start[k] + l; j < j1; j += kGradLanes) {
+    for (int j = j0 + l; j < j1; j += kGradLanes) {
       const GradRec r = m.grad[j];
-      double x = r.kind == MOD_HISTOSYS ? F[r.sample] : S[r.sample], y = 1.0;
-      if (r.kind == MOD_HISTOSYS) y = T[r.hs];
-      else if (r.kind == MOD_NORMSYS) y = fma(r.b, dg, r.a);
-      else x /= a;  // (one rounding; by the reciprocal it would be two)
-      g = fma(x, y, g);
+      const bool hs = r.kind == MOD_HISTOSYS;
+      g = fma(hs ? F[r.sample] : S[r.sample], hs ? T[r.hs] : fma(r.b, dg, r.a), g);
     }
   }
 #pragma unroll
@@ -457,7 +461,7 @@ struct GrowBuf {
 struct rf_binned {
   int32_t n_bins = 0, n_samples = 0, n_params = 0, n_mods = 0, n_entries = 0, n_hs = 0;
   rf::DevBuf bin0, nb, eofs, esample, nominal, smod_start, shs_start, shs, hs_param, hs_ofs, coef, tbase, g_sample,
-      bin_start, bin_entry, pmod_start, constrained, nominal_f, coef_f, coef_af, coef_bf, shs_k, shs_ofs, factor, grad;
+      bin_start, bin_entry, pmod_start, pmod_norm, constrained, nominal_f, coef_f, coef_af, coef_bf, shs_k, shs_ofs, factor, grad;
   rf::DevBuf counts, theta, out, flags, sets, io;
   GrowBuf work, scratch;  // intermediate results of the passes, of the expected counts
   rf::HostBuf h_out, h_flags, h_theta, h_sets, h_io;
@@ -642,7 +646,8 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   const int n_hs = (int)hs_param.size();
   // CSR lists: factor modifiers and histosys per sample, modifiers per
   // parameter (modifier order), the entries of each bin (sample order).
-  std::vector<int32_t> smod_start(n_samples + 1, 0), shs_start(n_samples + 1, 0), pmod_start(n_params + 1, 0);
+  std::vector<int32_t> smod_start(n_samples + 1, 0), shs_start(n_samples + 1, 0), pmod_start(n_params + 1, 0),
+      pmod_norm(n_params);
   for (int j = 0; j < n_mods; ++j) {
     (kind[j] == RF_MOD_HISTOSYS ? shs_start : smod_start)[msample[j] + 1]++;
     pmod_start[param[j] + 1]++;
@@ -660,6 +665,10 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
     else smod[sfill[msample[j]]++] = j;
     pmod[pfill[param[j]]++] = j;
   }
+  for (int k = 0; k < n_params; ++k)
+    pmod_norm[k] = (int32_t)(std::stable_partition(pmod.begin() + pmod_start[k], pmod.begin() + pmod_start[k + 1],
+                                                   [&](int32_t j) { return kind[j] == RF_MOD_NORMFACTOR; }) -
+                             pmod.begin());
   // transposed coefficients per sample
   std::vector<int64_t> tbase(n_samples);
   std::vector<int32_t> g_sample(shs.size());
@@ -726,7 +735,7 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
                   upload(m->shs, shs) && upload(m->hs_param, hs_param) && upload(m->hs_ofs, hs_ofs) &&
                   upload(m->coef, coef) && upload(m->tbase, tbase) && upload(m->g_sample, g_sample) &&
                   upload(m->bin_start, bin_start) && upload(m->bin_entry, bin_entry) &&
-                  upload(m->pmod_start, pmod_start) && upload(m->constrained, vcon);
+                  upload(m->pmod_start, pmod_start) && upload(m->pmod_norm, pmod_norm) && upload(m->constrained, vcon);
   m->smem = binned_smem(n_params, n_samples, n_bins);
   int dev_id = 0, max_optin = 0;
   cudaGetDevice(&dev_id);
@@ -779,6 +788,7 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   D.bin_start = (const int32_t*)m->bin_start.p;
   D.bin_entry = (const int32_t*)m->bin_entry.p;
   D.pmod_start = (const int32_t*)m->pmod_start.p;
+  D.pmod_norm = (const int32_t*)m->pmod_norm.p;
   D.constrained = (const int32_t*)m->constrained.p;
   D.factor = (const FactorRec*)m->factor.p;
   D.grad = (const GradRec*)m->grad.p;
