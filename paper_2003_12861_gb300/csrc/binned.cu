@@ -77,9 +77,7 @@ struct BinnedDev {
   const int32_t* smod_start;  // per sample: its normfactor / normsys modifiers (CSR, modifier order; `factor`)
   const int32_t* shs_start;   // per sample: its histosys modifiers (CSR, modifier order), as indices
   const int32_t* shs;         //   into the histosys arrays below
-  const int32_t* hs_param;    // per histosys: its parameter
-  const int64_t* hs_ofs;      // per histosys: a_i then b_i, nb each, in `coef`
-  const double* coef;
+  const double* coef;         // per histosys: a_i then b_i, nb each (at shs_ofs)
   // The same coefficients transposed per sample for the weighted sums:
   // sample s's histosys j (its j-th in shs order) at local bin i sits at
   // tbase[s] + i * (histosys of s) + j, in coef_af and coef_bf.
@@ -148,16 +146,21 @@ __device__ __forceinline__ void sample_factors(const BinnedDev& m, const double*
   __syncthreads();
 }
 
-// nu of every (sample, bin) entry in FP64 (for the expected counts).
+// nu of every (sample, bin) entry in FP64 (for the expected counts).  A block
+// waits for its chain of loads (a histosys's parameter and offset, then its
+// coefficients), so these are two levels, four at a time: one dataset of the
+// 28-channel model 355 -> 213 us, 1024 995 -> 894.
 __device__ __forceinline__ void entry_rates(const BinnedDev& m, const double* th, const double* gk, const double* F,
                                             double* nu_e) {
   for (int e = threadIdx.x; e < m.n_entries; e += kBinnedThreads) {
     const int s = m.esample[e], i = e - m.eofs[s], n = m.nb[s];
     double shape = m.nominal[e];
-    for (int j = m.shs_start[s]; j < m.shs_start[s + 1]; ++j) {
-      const int h = m.shs[j], k = m.hs_param[h];
-      const double* c = m.coef + m.hs_ofs[h] + i;
-      shape = fma(c[n], gk[k], fma(c[0], th[k], shape));
+    const int j1 = m.shs_start[s + 1];
+#pragma unroll 4
+    for (int j = m.shs_start[s]; j < j1; ++j) {
+      const int k = __ldg(m.shs_k + j);
+      const double* c = m.coef + __ldg(m.shs_ofs + j) + i;
+      shape = fma(__ldg(c + n), gk[k], fma(__ldg(c), th[k], shape));
     }
     nu_e[e] = F[s] * shape;
   }
@@ -460,7 +463,7 @@ struct GrowBuf {
 
 struct rf_binned {
   int32_t n_bins = 0, n_samples = 0, n_params = 0, n_mods = 0, n_entries = 0, n_hs = 0;
-  rf::DevBuf bin0, nb, eofs, esample, nominal, smod_start, shs_start, shs, hs_param, hs_ofs, coef, tbase, g_sample,
+  rf::DevBuf bin0, nb, eofs, esample, nominal, smod_start, shs_start, shs, coef, tbase, g_sample,
       bin_start, bin_entry, pmod_start, pmod_norm, constrained, nominal_f, coef_f, coef_af, coef_bf, shs_k, shs_ofs, factor, grad;
   rf::DevBuf counts, theta, out, flags, sets, io;
   GrowBuf work, scratch;  // intermediate results of the passes, of the expected counts
@@ -732,7 +735,7 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
                   upload(m->coef_af, pairs(coef_a)) && upload(m->coef_bf, pairs(coef_b)) &&
                   upload(m->bin0, vb0) && upload(m->nb, vnb) && upload(m->eofs, eofs) && upload(m->esample, esample) &&
                   upload(m->nominal, vnom) && upload(m->smod_start, smod_start) && upload(m->shs_start, shs_start) &&
-                  upload(m->shs, shs) && upload(m->hs_param, hs_param) && upload(m->hs_ofs, hs_ofs) &&
+                  upload(m->shs, shs) &&
                   upload(m->coef, coef) && upload(m->tbase, tbase) && upload(m->g_sample, g_sample) &&
                   upload(m->bin_start, bin_start) && upload(m->bin_entry, bin_entry) &&
                   upload(m->pmod_start, pmod_start) && upload(m->pmod_norm, pmod_norm) && upload(m->constrained, vcon);
@@ -774,8 +777,6 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   D.smod_start = (const int32_t*)m->smod_start.p;
   D.shs_start = (const int32_t*)m->shs_start.p;
   D.shs = (const int32_t*)m->shs.p;
-  D.hs_param = (const int32_t*)m->hs_param.p;
-  D.hs_ofs = (const int64_t*)m->hs_ofs.p;
   D.coef = (const double*)m->coef.p;
   D.tbase = (const int64_t*)m->tbase.p;
   D.g_sample = (const int32_t*)m->g_sample.p;
