@@ -90,3 +90,15 @@ def test_a_captured_pass_outlives_the_growth():
         assert np.array_equal(got[:, 0], want[0]) and np.array_equal(got[:, 1:], want[1])
     ref = m.nll_grad(more, more_th)
     assert np.array_equal(ref[0], grown[0]) and np.array_equal(ref[1], grown[1])
+
+
+def test_more_datasets_than_a_pass_takes():
+    spec = _one_bin()
+    m, one = api.BinnedModel(spec), api.BinnedModel(spec)
+    counts, th = _points(m, spec, 2 * 32768 + 5, 8)
+    nll, g = m.nll_grad(counts, th)
+    for t in (0, 1, 32767, 32768, 65535, 65536, 65540):
+        n, h = one.nll_grad(counts[t], th[t])
+        assert n[0] == nll[t] and np.array_equal(h[0], g[t]), t
+    back, gb = one.nll_grad(counts[::-1], th[::-1])
+    assert np.array_equal(back[::-1], nll) and np.array_equal(gb[::-1], g)
