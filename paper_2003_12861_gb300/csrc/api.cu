@@ -526,8 +526,10 @@ rf_status finish_data(rf_data* d) {
   d->chunks.resize(S);
   d->tree_base.resize(S);
   int64_t total = 0;
+  d->max_set = 0;
   for (int s = 0; s < S; ++s) {
     const int64_t n = d->offsets[s + 1] - d->offsets[s];
+    d->max_set = std::max(d->max_set, n);
     d->chunks[s] = (n + kChunk - 1) / kChunk;
     d->tree_base[s] = total;
     total += tree_nodes(d->chunks[s]);

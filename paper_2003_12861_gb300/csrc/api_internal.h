@@ -147,6 +147,7 @@ struct rf_data {
   std::vector<int64_t> offsets, chunks, tree_base;
   int64_t total_nodes = 0;
   int64_t total_chunks = 0;  // over all sets (parts_for)
+  int64_t max_set = 0;       // events of the largest set
   rf::DevBuf offsets_dev, tree_base_dev;
   rf::Workspace ws;
   rf::Plan all_plan;

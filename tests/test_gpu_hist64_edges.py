@@ -1,4 +1,5 @@
-"""hist64's bins on ranges near the smallest floats, against the FP64 definition."""
+"""hist64's bins on ranges near the smallest floats and with sets around the sizes
+at which its kernel changes form, against the FP64 definition."""
 import numpy as np
 import pytest
 
@@ -35,3 +36,26 @@ def test_ranges_near_the_smallest_floats(lo, hi, f32):
     api.hist64(m, api.Data.upload(m, [x]), 0, out)
     torch.cuda.synchronize()
     assert np.array_equal(out.cpu().numpy()[0], _fractions(x, lo, hi))
+
+
+# 511 and 512: the blocks' size; 1023 and 1024: one copy of the counters or 16;
+# 2 x 16384 per set on average: one block a set or two
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("sizes", [[511, 0, 63], [512, 1, 0, 65], [1023, 1024, 3], [1], [300] * 700, [40000, 0, 5, 100],
+                                   [32767], [32768], [70000, 20000, 8304], [5, 98299]])
+def test_set_sizes_around_the_kernels_forms(sizes, f32):
+    import torch
+
+    lo, hi = 0.0, 10.0
+    m = _model(lo, hi)
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    x = np.random.default_rng(int(off[-1])).exponential(1.5, off[-1])
+    x = x.astype(np.float32) if f32 else x
+    out = torch.full((len(sizes), 64), 3.0, dtype=torch.float32, device="cuda")
+    api.hist64(m, api.Data.upload(m, [x], offsets=off), 0, out)
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    for s in range(len(sizes)):
+        part = x[off[s]:off[s + 1]]
+        want = _fractions(part, lo, hi) if len(part) else np.zeros(64, dtype=np.float32)
+        assert np.array_equal(got[s], want), s
