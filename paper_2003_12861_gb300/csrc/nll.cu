@@ -580,7 +580,6 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
   constexpr bool kKeep = kGrad && kKept;
   double w1[kKeep ? kMaxPdf : 1];             // per node: u, or the unnormalised value
   double w2[kKeep && kFull ? kMaxPdf : 1];    // GAUSSEXP: exp(-u^2/2)
-  double f1[kKeep && kFull ? kMaxPdf : 1];    // and the convolution
   double dex[kGrad && kExpr ? kMaxSlots : 1]; // EXPR: derivatives by slot
   const int N = n1 < 0 ? P.n_pdf : n1;
   for (int n = n0; n < N; ++n) {
@@ -607,10 +606,7 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
           const double g = kGrad || right ? mt.exp_(-0.5 * u * u) : 0.0;
           const double w = right ? g : mt.exp_(s * (0.5 * s - u));
           f = 0.5 * w * mt.tail(z, right);
-          if constexpr (kKeep) {
-            w2[n] = g;
-            f1[n] = f;
-          }
+          if constexpr (kKeep) w2[n] = g;
         }
         v[n] = f * c[4];
         break;
@@ -717,11 +713,11 @@ __device__ bool eval_generic(const Program& P, const double* __restrict__ C, con
           g[s0 + 1] += w * (it - c[6]);
           g[s0 + 2] += w * (sit - c[7]);
         } else {  // df = f dA - exp(-u^2/2)/sqrt(pi) dz, with no division by f
-          const double w = a * c[4], f = kKeep ? f1[n] : v[n] / c[4];
-          const double h = (kKeep ? w2[n] : exp(-0.5 * u * u)) * kInvSqrt2Pi;
-          g[s0] += w * (f * (sit * (u - s) - c[5]) + h * sit);
-          g[s0 + 1] += w * (f * (it - c[6]) - h * c[1]);
-          g[s0 + 2] += w * (f * (sit - c[7]) - h * (it + u * c[1]));
+          // (1/I on f and h, not on a: a / I would overflow where f is subnormal)
+          const double h = (kKeep ? w2[n] : exp(-0.5 * u * u)) * kInvSqrt2Pi * c[4];
+          g[s0] += a * (v[n] * (sit * (u - s) - c[5]) + h * sit);
+          g[s0 + 1] += a * (v[n] * (it - c[6]) - h * c[1]);
+          g[s0 + 2] += a * (v[n] * (sit - c[7]) - h * (it + u * c[1]));
         }
         break;
       }
