@@ -41,21 +41,22 @@ __device__ __forceinline__ double quotient(double t, const Divisor& d) {
 // The program's value at x and, for kDeriv, its derivatives in the node's
 // parameters (forward mode), df[0..n_par).  par: the node's parameter values.
 // Returns 0 if the value is finite and in the program's domain (no log or pow
-// of a value <= 0, no division by 0), with kDeriv plus 2 if some derivative
-// is not finite (df is then NaN throughout); 1 otherwise (df not written).
+// of a value <= 0, no division by 0), with kDeriv 2 if some derivative is not
+// finite; 1 otherwise (df not written).
 //
 // An FP64 warp instruction occupies its sub-partition's unit for some 64
 // cycles, an integer one for 1, so the interpretation is free and only the
 // FP64 operations count: each stack entry carries a mask of the parameters
 // that it depends on, and only their tangents are computed.  The others'
 // are zero; where arithmetic with that zero would give NaN (times an
-// infinity), the derivatives are marked not finite all the same.
+// infinity), all derivatives are NaN all the same.  One that leaves the finite
+// range by itself leaves the others as they are.
 template <bool kDeriv, class M = LibMath>
 __device__ __forceinline__ int expr_eval(const Program& P, const PNode& q, const double* par, double x, double* f,
                                          double* df, const M& mt = M()) {
   double v[kExprStack], d[kDeriv ? kExprStack : 1][kMaxPar];
   unsigned act[kDeriv ? kExprStack : 1];
-  bool wild = false;  // a tangent left the finite range
+  bool wild = false;  // a value that tangents are multiplied with left the finite range
   int sp = 0;
   const int32_t* ops = P.ex_ops + q.ex_op0;
   const double* cs = P.ex_consts + q.ex_c0;
@@ -154,14 +155,12 @@ __device__ __forceinline__ int expr_eval(const Program& P, const PNode& q, const
   *f = v[0];
   if (not_finite(v[0])) return 1;
   if constexpr (kDeriv) {
+    bool any = false;
     for (int k = 0; k < q.n_par; ++k) {
-      df[k] = (act[0] >> k & 1u) ? d[0][k] : 0.0;
-      wild |= not_finite(df[k]);
+      df[k] = wild ? NAN : (act[0] >> k & 1u) ? d[0][k] : 0.0;
+      any |= not_finite(df[k]);
     }
-    if (wild && q.n_par > 0) {
-      for (int k = 0; k < q.n_par; ++k) df[k] = NAN;
-      return 2;
-    }
+    if (any) return 2;
   }
   return 0;
 }
