@@ -103,6 +103,12 @@ bool build_plan(const rf_data* d, const std::vector<int32_t>& sets, Plan* plan) 
   }
   plan->n_active = (int)sets.size();
   plan->n_items = (int)items.size();
+  for (int l = 0; l < 5; ++l) {
+    const int64_t part = kChunk >> l;
+    int64_t n = 0;
+    for (int32_t s : sets) n += (d->offsets[s + 1] - d->offsets[s] + part - 1) / part;
+    plan->n_units[l] = (int32_t)std::min<int64_t>(n, INT32_MAX);
+  }
   plan->host_sets = sets;
   if (!plan->sets.ensure(sizeof(int32_t) * std::max<size_t>(1, sets.size()))) return false;
   if (!plan->items.ensure(sizeof(int2) * std::max<size_t>(1, items.size()))) return false;
@@ -183,6 +189,8 @@ Pass make_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* d_
   p.part_fb = (double*)w.part_fb.p;
   p.part_info = (int32_t*)w.part_info.p;
   p.parts = parts_for(d->total_chunks, m->m.shape);
+  for (int l = 0; l < 5; ++l)
+    if (p.parts == 1 << l) p.n_units = plan.n_units[l];
   p.pairs = nullptr;
   return p;
 }
@@ -201,6 +209,7 @@ bool launch_pass(const rf_model* m, rf_data* d, const Plan& plan, const double* 
                  const double* theta1) {
   Pass pass = make_pass(m, d, plan, d_theta, d_out, d_flags, grad);
   pass.dyn = dyn;
+  if (dyn) pass.n_units = 0;  // (the device compacts the plan)
   pass.flags_out = flags_out;
   if (theta1) {
     pass.n_theta1 = m->m.prog.n_free;
@@ -721,6 +730,7 @@ extern "C" rf_status rf_nll_grad_stream(const rf_model* m, rf_data* d, const voi
     Pass seg = pass;
     seg.items = (const int2*)plan.items.p + i0;
     seg.n_items = (int32_t)(i1 - i0);
+    seg.n_units = 0;
     seg.counter = pass.counter + k;
     launch_events(m->m.prog, m->m.shape, cols, seg, m->m.threads_per_block, m->m.blocks_per_sm, sm_count(), cs);
   }

@@ -38,6 +38,7 @@ struct Plan {
   DevBuf sets, items;
   std::vector<int32_t> host_sets;
   int32_t n_active = 0, n_items = 0;
+  int32_t n_units[5] = {};  // parts of the items that have events, with 1, 2, 4, 8, 16 parts a chunk
 };
 
 // Segments of the streamed host-column pass (rf_nll_grad_stream).

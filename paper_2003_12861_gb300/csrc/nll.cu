@@ -948,20 +948,21 @@ __device__ __forceinline__ void warp_sums(const double* acc, int Q, double* buf,
   }
 }
 
-// Ends a work unit: the block's sums (lanes, then warps in a fixed order) go
-// to the chunk's level-0 tree node if the unit is the whole chunk, otherwise
-// to the part's record; the block that completes the chunk's last part
-// merges the parts in part order.  Then the climb up the tree.
+// Ends a work unit, the part-th of the `parts` parts of its chunk that have
+// events: the block's sums (lanes, then warps in a fixed order) go to the
+// chunk's level-0 tree node if the unit is the only one, otherwise to the
+// part's record; the block that completes the chunk's last part merges the
+// parts in part order.  Then the climb up the tree.
 __device__ void finish_unit(const Program& P, const Pass& pass, Smem& sm, const double* acc, int bad, int set,
-                            int chunk, int part, int64_t n_events) {
+                            int chunk, int part, int parts, int64_t n_events) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int Q = pass.Q, parts = pass.parts;
+  const int Q = pass.Q;
   warp_sums(acc, Q, (double*)sm.queue[warp], sm.wsum[warp], lane);
   bad = warp_sum_int(bad);
   if (lane == 0) sm.wbad[warp] = bad;
   __syncthreads();
   const int64_t node = pass.tree_base[set] + chunk;
-  const int64_t rec = node * parts + part;
+  const int64_t rec0 = node * pass.parts, rec = rec0 + part;
   double* dst = parts == 1 ? pass.tree + node * 2 * Q : pass.part_fb + rec * 2 * Q;
   if (tid < Q) {
     Pair a = merge({sm.wsum[0][tid], 0.0}, {sm.wsum[1][tid], 0.0});
@@ -984,7 +985,7 @@ __device__ void finish_unit(const Program& P, const Pass& pass, Smem& sm, const 
     if (!sm.last) return;
     __threadfence();
     if (tid < Q) {
-      const double* p = pass.part_fb + node * parts * 2 * Q + tid;
+      const double* p = pass.part_fb + rec0 * 2 * Q + tid;
       Pair r{__ldcg(p), __ldcg(p + Q)};
       for (int i = 1; i < parts; ++i) r = merge(r, {__ldcg(p + i * 2 * Q), __ldcg(p + i * 2 * Q + Q)});
       pass.tree[node * 2 * Q + tid] = r.s;
@@ -992,7 +993,7 @@ __device__ void finish_unit(const Program& P, const Pass& pass, Smem& sm, const 
     }
     if (tid == 0) {
       int b = 0;
-      for (int i = 0; i < parts; ++i) b += __ldcg(pass.part_info + node * parts + i);
+      for (int i = 0; i < parts; ++i) b += __ldcg(pass.part_info + rec0 + i);
       pass.tree_bad[node] = b;
     }
   }
@@ -1006,7 +1007,12 @@ __device__ void finish_unit(const Program& P, const Pass& pass, Smem& sm, const 
 // (ballot order) and evaluated after the fast pass, so the warp stays
 // converged; the lane order of additions is still fixed by the data alone.
 // The next unit is claimed after the unit's events, when the other blocks
-// have had their share.
+// have had their share.  Units run part by part over the items, and the grid
+// has a block for each that has events (launch_events): with a block for each
+// of a small set's empty parts too, the sets' units met on half of the SMs and
+// their empty ones ran the whole end of a unit (Gauss + exponential, 400 sets
+// of 1500 events 152 us before there were parts, 198 with them, 125 so; 260
+// sets 125, 173, 115; 260 of 200 events 77, 88, 63).
 // Bound by the FP64 unit.  First with the split into parts, one evaluation of
 // a program per event and the values kept for the gradient pass, then with
 // the functions of fp64_math.cuh: decay model 1e4 events 203 -> 41 -> 39 us,
@@ -1018,7 +1024,7 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
   __shared__ Smem sm;
   __shared__ double2 exp_tab[256];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_units = (pass.dyn ? pass.dyn[1] : pass.n_items) * pass.parts;
+  const int n_items = pass.dyn ? pass.dyn[1] : pass.n_items, n_units = n_items * pass.parts;
   if (n_units == 0) return;
   for (int i = tid; i < 256; i += kLanes) exp_tab[i] = ((const double2*)kExp64)[i];
   const TableMath mt{exp_tab};
@@ -1026,13 +1032,24 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
   const int per_lane = kPerLane / pass.parts;
   if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
   __syncthreads();
-  while (true) {
-    const int u = sm.item;
-    if (u >= n_units) break;
-    const int it = u / pass.parts, part = u % pass.parts;
+  int u = sm.item;
+  while (u < n_units) {
+    const int part = u / n_items, it = u - part * n_items;
     const int set = pass.items[it].x, chunk = pass.items[it].y;
     const int64_t s_begin = pass.offsets[set], s_end = pass.offsets[set + 1];
-    const int64_t base = s_begin + (int64_t)chunk * kChunk + part * (per_lane * kLanes);
+    // A part without events (a set's last chunk is short, a small set's only one
+    // very) is no part of its chunk: it would add zeros.
+    const int per_part = per_lane * kLanes;
+    const int64_t chunk0 = s_begin + (int64_t)chunk * kChunk;
+    const int parts = ((int)min((int64_t)kChunk, s_end - chunk0) + per_part - 1) / per_part;
+    if (part >= parts) {
+      __syncthreads();
+      if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
+      __syncthreads();
+      u = sm.item;
+      continue;
+    }
+    const int64_t base = chunk0 + part * per_part;
     for (int i = tid; i < P.n_const; i += kLanes) sm.C[i] = pass.consts[(size_t)set * P.n_const + i];
     __syncthreads();
     double acc[kQMax];
@@ -1063,8 +1080,9 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
     if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
     acc[0] += logprod64_log(L);
     __syncwarp();
-    finish_unit(P, pass, sm, acc, bad, set, chunk, part, s_end - s_begin);
+    finish_unit(P, pass, sm, acc, bad, set, chunk, part, parts, s_end - s_begin);
     __syncthreads();
+    u = sm.item;
   }
 }
 
@@ -1440,7 +1458,8 @@ void launch_events(const Program& P, Shape shape, const Columns& cols, const Pas
   const int bps = blocks_per_sm > 0 ? blocks_per_sm : 8;
   int grid = n_sm * bps;
   const Shape sh = (pass.ff_shape != SHAPE_GENERIC && pass.ffc) ? shape : SHAPE_GENERIC;
-  const int64_t units = (int64_t)pass.n_items * pass.parts;
+  const int64_t units =
+      sh == SHAPE_GENERIC && pass.n_units > 0 ? pass.n_units : (int64_t)pass.n_items * pass.parts;
   if (grid > units) grid = (int)units;
   note_launches(1, st);
   timing_begin(st);

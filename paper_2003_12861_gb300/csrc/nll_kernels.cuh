@@ -21,6 +21,7 @@ struct Pass {
   int32_t n_active;
   const int2* items;        // (set, chunk) work items of the active sets
   int32_t n_items;
+  int32_t n_units;          // generic kernel: of its n_items x parts units, those that have events (0: not known)
   const int64_t* tree_base; // per set: first node of its reduction tree
   const double* theta;      // n_sets x n_free
   double* consts;           // n_sets x n_const

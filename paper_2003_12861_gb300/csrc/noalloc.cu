@@ -193,6 +193,7 @@ extern "C" rf_status rf_nll_grad_noalloc(const rf_model* m, const void* const* d
   pass.part_fb = (double*)(base + L.part_fb);
   pass.part_info = (int32_t*)(base + L.part_info);
   pass.parts = parts_for(chunks, m->m.shape);
+  pass.n_units = (int32_t)((n_events + kChunk / pass.parts - 1) / (kChunk / pass.parts));
   launch_param_point(P, pass, st);
   launch_events(P, m->m.shape, cols, pass, m->m.threads_per_block, m->m.blocks_per_sm, sm_count(), st);
   return cuda_ok(cudaGetLastError(), "rf_nll_grad_noalloc launch") ? RF_OK : RF_E_CUDA;
