@@ -340,7 +340,8 @@ def transcendental_ceiling(api, model_spec, slow_fraction, n_events, bytes_per_e
     return alu, hbm, basis
 
 
-KERNEL_SOURCES = ["nll.cu", "nll_ff.cuh", "k1_ff.cuh", "ff.cuh", "ff_tables.h", "nll_kernels.cuh", "rf_internal.h", "expr.cuh"]
+KERNEL_SOURCES = ["nll.cu", "nll_ff.cuh", "k1_ff.cuh", "ff.cuh", "ff_tables.h", "nll_kernels.cuh", "rf_internal.h", "expr.cuh",
+                  "fp64_math.cuh", "fp64_tables.h"]
 
 
 def kernel_digest():

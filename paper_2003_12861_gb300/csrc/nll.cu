@@ -1133,17 +1133,18 @@ __device__ __forceinline__ bool ff_lane_writes(int lane) {
 __host__ __device__ constexpr int pow2_at_least(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : 16; }
 
 // Float-float fused event kernel of a specialised shape.  Persistent blocks
-// of 128 threads take work units from the counter: unit u is part u % 4 of
-// work item u / 4 (a quarter of a 4096-event chunk, 8 events per lane), so
-// the last round of units is short.  Per lane the shape's moments are summed
-// in float-float; events in the decay resolution region are queued per warp
-// (ballot order) and evaluated after the fast pass by all the block's
-// threads; events outside the
+// of 128 threads take work units from the counter: with pass.parts = 1, 2 or
+// 4 parts a chunk (parts_for), unit u is part u % parts of work item
+// u / parts, 32 / parts events per lane of a 4096-event chunk.  Per lane the
+// shape's moments are summed in float-float; a lane marks its events in the
+// decay resolution region in a bit mask, and after the fast pass all the
+// block's threads share them out and evaluate them; events outside the
 // float-float range take the FP64 interpreter (FP64 sums).  At the end of a
-// part the warps' moments are merged in fixed order and stored as the part's
-// record; the block that completes the chunk's last part (arrival ticket)
-// merges the four records in part order, maps the moments to (sum log p,
-// slot gradients) with the set's matrix K and climbs the reduction tree.
+// part the warps' moments are merged in fixed order; with several parts they
+// are stored as the part's record and the block that completes the chunk's
+// last part (arrival ticket) merges the records in part order.  The chunk's
+// moments are mapped to (sum log p, slot gradients) with the set's matrix K,
+// then the climb up the reduction tree.
 // Every sum has a fixed order, so the result does not depend on the launch.
 template <int kShape, bool kGrad, bool kF32>
 __global__ void __launch_bounds__(kLanes, ff_min_blocks(kShape)) events_ff(const __grid_constant__ Program P,
