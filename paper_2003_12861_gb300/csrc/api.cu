@@ -64,6 +64,27 @@ bool DevBuf::ensure(size_t b) {
   return true;
 }
 
+bool GrowBuf::ensure(size_t b) {
+  if (b <= bytes && p) return true;
+  kept_.emplace_back();
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const bool ok = kept_.back().ensure(b);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (!ok) {
+    kept_.pop_back();
+    return false;
+  }
+  p = kept_.back().p;
+  bytes = kept_.back().bytes;
+  return true;
+}
+void GrowBuf::release() {
+  kept_.clear();
+  p = nullptr;
+  bytes = 0;
+}
+
 HostBuf::~HostBuf() {
   if (p) cudaFreeHost(p);
 }

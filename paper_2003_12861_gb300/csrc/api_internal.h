@@ -5,6 +5,7 @@
 
 #include <cstdint>
 #include <functional>
+#include <list>
 #include <string>
 #include <vector>
 
@@ -21,6 +22,22 @@ struct DevBuf {
   ~DevBuf();
   bool ensure(size_t b);
   void release();
+};
+
+// A buffer that keeps what it had when it grows, as queued work and captured
+// graphs use it.  The stream may be capturing: the allocation is no part of
+// that.  Without memory it stays as it was.
+struct GrowBuf {
+  void* p = nullptr;
+  size_t bytes = 0;
+  GrowBuf() = default;
+  GrowBuf(const GrowBuf&) = delete;
+  GrowBuf& operator=(const GrowBuf&) = delete;
+  bool ensure(size_t b);
+  void release();
+
+ private:
+  std::list<DevBuf> kept_;  // the last one is in use
 };
 
 struct HostBuf {
@@ -48,9 +65,10 @@ constexpr int kMaxSegments = 16;
 constexpr int kCompStreams = 4;
 
 // A dataset's evaluation buffers, grown to the largest that a model evaluated
-// on it needs (ensure_workspace; sizes in workspace.h).
+// on it needs (ensure_workspace; sizes in workspace.h).  A captured pass of one
+// model stays valid when another one grows them.
 struct Workspace {
-  DevBuf consts, theta, out, flags, tree, tree_bad, tickets, counter, slow, ffc, part_m, part_fb, part_info;
+  GrowBuf consts, theta, out, flags, tree, tree_bad, tickets, counter, slow, ffc, part_m, part_fb, part_info;
   // work and slow-event counters of passes that may run concurrently on
   // other streams (launch_pass with slot >= 0)
   DevBuf slot_counter, slot_slow;

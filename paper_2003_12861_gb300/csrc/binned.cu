@@ -35,7 +35,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <list>
 #include <vector>
 
 #include "api_internal.h"
@@ -442,31 +441,12 @@ __global__ void __launch_bounds__(kBinnedThreads) binned_expected_kernel(const B
 
 // ---------------------------------------------------------------- handle
 
-// A buffer that grows and keeps what it had (at most as much again, if it
-// grows at least twofold), as queued work and captured graphs use it.  The
-// stream may be capturing: the allocation is no part of that.
-struct GrowBuf {
-  std::list<rf::DevBuf> kept;  // the last one is in use
-  void* p() const { return kept.empty() ? nullptr : kept.back().p; }
-  size_t bytes() const { return kept.empty() ? 0 : kept.back().bytes; }
-  bool grow(size_t b) {
-    if (b <= bytes()) return true;
-    kept.emplace_back();
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    const bool ok = kept.back().ensure(b);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (!ok) kept.pop_back();
-    return ok;
-  }
-};
-
 struct rf_binned {
   int32_t n_bins = 0, n_samples = 0, n_params = 0, n_mods = 0, n_entries = 0, n_hs = 0;
   rf::DevBuf bin0, nb, eofs, esample, nominal, smod_start, shs_start, shs, coef, tbase, g_sample,
       bin_start, bin_entry, pmod_start, pmod_norm, constrained, nominal_f, coef_f, coef_af, coef_bf, shs_k, shs_ofs, factor, grad;
   rf::DevBuf counts, theta, out, flags, sets, io;
-  GrowBuf work, scratch;  // intermediate results of the passes, of the expected counts
+  rf::GrowBuf work, scratch;  // intermediate results of the passes, of the expected counts
   rf::HostBuf h_out, h_flags, h_theta, h_sets, h_io;
   rf::BinnedDev dev{};
   rf::BinnedScratch ws{};
@@ -522,9 +502,9 @@ bool reserve_sets(rf_binned* m, int n) {
   const int most = held((size_t)256 << 20);
   if (m->cap > 0 && std::min(n, most) <= m->cap) return true;
   const int cap = std::min(most, n > 0 ? std::max(n, 2 * m->cap) : held((size_t)8 << 20));
-  if (!m->work.grow(per_set * (size_t)cap)) return false;
+  if (!m->work.ensure(per_set * (size_t)cap)) return false;
   m->cap = cap;
-  char* p = (char*)m->work.p();  // (16-byte items first)
+  char* p = (char*)m->work.p;  // (16-byte items first)
   auto take = [&](size_t bytes) {
     char* q = p;
     p += bytes * (size_t)cap;
@@ -760,7 +740,7 @@ rf_status rf_binned_create(int32_t n_bins, int32_t n_samples, const int32_t* bin
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, binned_expected_kernel, kBinnedThreads, m->smem);
   m->grid = sm_count() * std::max(1, per_sm);
-  if (!ok || !m->scratch.grow(sizeof(double) * (size_t)total) || !reserve_sets(m, 0)) {
+  if (!ok || !m->scratch.ensure(sizeof(double) * (size_t)total) || !reserve_sets(m, 0)) {
     delete m;
     return RF_E_OOM;
   }
@@ -885,12 +865,12 @@ rf_status rf_binned_expected(rf_binned* m, int32_t n_sets, const double* d_theta
   // as many as there is room for.
   const size_t per_block = sizeof(double) * (size_t)m->n_entries;
   int grid = std::min(n_sets, m->grid);
-  if (m->scratch.bytes() < per_block * (size_t)grid)
-    m->scratch.grow(per_block * std::min((size_t)m->grid, std::max((size_t)grid, 2 * m->scratch.bytes() / per_block)));
-  grid = (int)std::min((size_t)grid, m->scratch.bytes() / per_block);
+  if (m->scratch.bytes < per_block * (size_t)grid)
+    m->scratch.ensure(per_block * std::min((size_t)m->grid, std::max((size_t)grid, 2 * m->scratch.bytes / per_block)));
+  grid = (int)std::min((size_t)grid, m->scratch.bytes / per_block);
   note_launches(1, (cudaStream_t)stream);
   binned_expected_kernel<<<grid, kBinnedThreads, m->smem, (cudaStream_t)stream>>>(m->dev, n_sets, d_theta, d_nu,
-                                                                                  (double*)m->scratch.p());
+                                                                                  (double*)m->scratch.p);
   return cuda_ok(cudaGetLastError(), "binned launch") ? RF_OK : RF_E_CUDA;
 }
 
