@@ -185,7 +185,10 @@ rf_status rf_data_offsets(const rf_data* d, int64_t* out);
  * "the probability of observing each event"), non-extended.  theta and nll
  * are HOST arrays (n_sets x n_free, n_sets).  The sum is deterministic: it
  * is a fixed tree over 4096-event chunks (in-chunk lane sums, then
- * compensated two-sum merges), independent of launch shape.  A set with an
+ * compensated two-sum merges), independent of launch shape.  How many parts a
+ * chunk is summed in follows from the chunks of the whole dataset, so the last
+ * bits of a set's sums may differ between datasets (a batch, a set alone, a
+ * shard) that hold the same events.  A set with an
  * event whose pdf is <= 0 or not finite gets nll = +inf and the call returns
  * RF_E_DOMAIN.  Synchronous on `stream`. */
 rf_status rf_nll(const rf_model* m, const rf_data* d, const double* theta, double* nll, void* stream);
@@ -218,8 +221,8 @@ rf_status rf_nll_chunks(const rf_model* m, const rf_data* d, const double* theta
  * (bitwise), so threads_per_block accepts 0 or 128 only.  The tunable
  * dimension is blocks_per_sm, the resident blocks per SM of the persistent
  * grid (1..32; 0 = library choice).  The work unit (a whole 4096-event chunk,
- * or a quarter chunk for datasets of fewer than 1024 chunks) is fixed by
- * the dataset for the same reason. */
+ * or an equal part of one, down to 256 events, for a dataset of few chunks) is
+ * fixed by the dataset and the model's kernel for the same reason. */
 rf_status rf_set_launch(rf_model* m, int32_t threads_per_block, int32_t blocks_per_sm);
 
 /* Autotuner: times `passes` NLL+gradient passes over `d` for every resident

@@ -16,8 +16,9 @@
 //
 // (One block per dataset, each reading every coefficient for itself and waiting
 // for it, took 490 us for one dataset of the 28-channel model and 1500 us for
-// 1024; this takes 76 and 856 us: the float-float loops 0.29 ms each, at about
-// 60 % of the FP32 pipe's rate, the bins' FP64 division and logarithm 0.13 ms.)
+// 1024; this takes 58 and 834 us a call: the float-float loops 0.29 ms each, at
+// about 60 % of the FP32 pipe's rate, the bins' FP64 division and logarithm
+// 0.13 ms.)
 // A pass is five chained kernels over (dataset, work) grids -- parameters and
 // sample factors, entry rates, bins, weighted sums, gradient and NLL -- so one
 // dataset fills as many SMs as its work can, and many datasets share every
@@ -792,8 +793,8 @@ rf_status rf_binned_nll_grad_async(rf_binned* m, int32_t n_sets, const double* d
   return launch_binned(m, n_sets, d_counts, d_theta, d_out, d_flags, (cudaStream_t)stream);
 }
 
-// Up to this many bytes of counts, parameters and results (some ten datasets
-// of 1400 bins) a host call goes through one pinned buffer: one dataset of
+// Up to this many bytes of counts, parameters and results (17 datasets of 1400
+// bins and 256 parameters) a host call goes through one pinned buffer: one dataset of
 // 1400 bins and 256 parameters 76 -> 58 us.
 constexpr size_t kStagedBytes = size_t(256) << 10;
 

@@ -3,9 +3,9 @@
 // the number of FP64 operations: a table look-up (integer and shared-memory
 // work, free beside them) takes the place of most of a polynomial.  Decay
 // model on 4e6 events 705 -> 601 us, program model on 1e6 355 -> 329.
-// Largest and mean error in units in the last place, here / CUDA's: exp
-// 0.55, 0.25 / 0.76, 0.25; erfc on [-7.5, 0] 0.54, 0.19 / 1.36, 0.21; erfcx
-// on [0, 9.5] 1.27, 0.27 / 1.96, 0.38.
+// Largest and mean error in units in the last place, here (from the tables) /
+// CUDA's: exp 0.58, 0.25 / 0.76, 0.25; erfc on [-7, 0] 0.55, 0.21 / 1.36, 0.21;
+// erfcx on [0, 8] 0.61, 0.25 / on [0, 9.5] 1.96, 0.38.
 #pragma once
 
 #include <cuda_runtime.h>

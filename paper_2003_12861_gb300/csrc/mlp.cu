@@ -438,7 +438,7 @@ struct ReduceArgs {
   int n_items;
   const double* loss;
   int n_loss;
-  double inv_n;  // (a division by n below)
+  double n;      // targets: the loss is the sum over them divided by n
   float* out;    // loss, flag
 };
 __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ ReduceArgs a) {
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Red
       __syncthreads();
     }
     if (tid == 0) {
-      a.out[0] = (float)(red[0] / a.inv_n);
+      a.out[0] = (float)(red[0] / a.n);
       reinterpret_cast<int*>(a.out)[1] = g_gemm_timeout;
     }
     return;
@@ -644,8 +644,8 @@ GemmArgs forward_args(rf_mlp* n, int l, const float* a_in, float* out, int batch
   return g;
 }
 
-// y = net(x): the layers' activations alternate between two halves of acts
-// (the pre-activations are not kept); the last layer writes y.
+// y = net(x): each layer's activations follow the one before in acts (the
+// pre-activations are not kept); the last layer writes y.
 void mlp_forward(rf_mlp* n, const float* x, int batch, float* y, cudaStream_t st) {
   const int L = (int)n->dims.size() - 1;
   const float* a_in = x;
@@ -735,7 +735,7 @@ rf_status mlp_loss_grad(rf_mlp* n, const float* x, const float* t, int batch, fl
   }
   r.loss = (const double*)n->sq.p;
   r.n_loss = ((batch + TM - 1) / TM) * ((no_last + TN - 1) / TN);
-  r.inv_n = (double)cnt;
+  r.n = (double)cnt;
   r.out = out;
   launch_chained(reduce_kernel, dim3(block + 1), 256, 0, st, r);
   return cuda_ok(cudaGetLastError(), "mlp launch") ? RF_OK : RF_E_CUDA;
