@@ -1012,7 +1012,7 @@ __device__ void finish_unit(const Program& P, const Pass& pass, Smem& sm, const 
 // of a small set's empty parts too, the sets' units met on half of the SMs and
 // their empty ones ran the whole end of a unit (Gauss + exponential, 400 sets
 // of 1500 events 152 us before there were parts, 198 with them, 125 so; 260
-// sets 125, 173, 115; 260 of 200 events 77, 88, 63).
+// sets 125, 173, 112; 260 of 200 events 77, 88, 63).
 // Bound by the FP64 unit.  First with the split into parts, one evaluation of
 // a program per event and the values kept for the gradient pass, then with
 // the functions of fp64_math.cuh: decay model 1e4 events 203 -> 41 -> 39 us,
@@ -1030,7 +1030,13 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
   const TableMath mt{exp_tab};
   pdl_wait();
   const int per_lane = kPerLane / pass.parts;
-  if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
+  // With several parts a block's first unit is its own number, and the units'
+  // order is that of the blocks on the SMs: claimed, large and small parts met
+  // by chance (260 sets of 1500 events, Gauss + exponential 120 -> 112 us,
+  // program model 306 -> 275).  Whole chunks are claimed from the first one on
+  // (4e6 events 2 % slower otherwise).
+  const int first = pass.parts > 1 ? (int)gridDim.x : 0;
+  if (tid == 0) sm.item = first > 0 ? (int)blockIdx.x : atomicAdd(pass.counter, 1);
   __syncthreads();
   int u = sm.item;
   while (u < n_units) {
@@ -1044,7 +1050,7 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
     const int parts = ((int)min((int64_t)kChunk, s_end - chunk0) + per_part - 1) / per_part;
     if (part >= parts) {
       __syncthreads();
-      if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
+      if (tid == 0) sm.item = first + atomicAdd(pass.counter, 1);
       __syncthreads();
       u = sm.item;
       continue;
@@ -1077,7 +1083,7 @@ __global__ void __launch_bounds__(kLanes) events_generic(const __grid_constant__
       for (int c = 0; c < P.n_obs; ++c) x[c] = load_col(cols, c, e);
       eval_generic<true, kGrad, kExpr>(P, sm.C, x, acc, L, &bad, 0, -1, mt);
     }
-    if (tid == 0) sm.item = atomicAdd(pass.counter, 1);
+    if (tid == 0) sm.item = first + atomicAdd(pass.counter, 1);
     acc[0] += logprod64_log(L);
     __syncwarp();
     finish_unit(P, pass, sm, acc, bad, set, chunk, part, parts, s_end - s_begin);
