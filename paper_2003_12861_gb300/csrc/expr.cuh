@@ -155,12 +155,15 @@ __device__ __forceinline__ int expr_eval(const Program& P, const PNode& q, const
   *f = v[0];
   if (not_finite(v[0])) return 1;
   if constexpr (kDeriv) {
-    bool any = false;
-    for (int k = 0; k < q.n_par; ++k) {
-      df[k] = wild ? NAN : (act[0] >> k & 1u) ? d[0][k] : 0.0;
-      any |= not_finite(df[k]);
+    if (wild && q.n_par > 0) {
+      for (int k = 0; k < q.n_par; ++k) df[k] = NAN;
+      return 2;
     }
-    if (any) return 2;
+    for (int k = 0; k < q.n_par; ++k) {
+      df[k] = (act[0] >> k & 1u) ? d[0][k] : 0.0;
+      wild |= not_finite(df[k]);
+    }
+    if (wild && q.n_par > 0) return 2;
   }
   return 0;
 }
